@@ -658,24 +658,6 @@ cudaError_t launch_factor_t(const FactorParamsT<double> &p, int njobs, cudaStrea
   return cudaGetLastError();
 }
 
-template <int MINB>
-cudaError_t launch_factor_c(const FactorParamsT<double> &p, int njobs, cudaStream_t s) {
-  if (p.nc <= 16) return launch_factor_t<1, MINB>(p, njobs, s);
-  if (p.nc <= 32) return launch_factor_t<2, MINB>(p, njobs, s);
-  if (p.nc <= 64) return launch_factor_t<4, MINB>(p, njobs, s);
-  return launch_factor_t<8, MINB>(p, njobs, s);
-}
-
-cudaError_t launch_factor_any(const FactorParamsT<double> &p, int njobs, int ctas_per_sm, cudaStream_t s) {
-  if (njobs <= 0) return cudaSuccess;
-  // up to 16 columns (one column slot per half-warp) a step keeps at most half of a CTA's
-  // worker warps busy: the 64-register build lets a fourth CTA join where its tile fits
-  // (the plan, made for three, is unchanged)
-  if (ctas_per_sm >= 3 && p.nc <= 16) return launch_factor_t<1, 4>(p, njobs, s);
-  if (ctas_per_sm >= 3) return launch_factor_c<3>(p, njobs, s);
-  return launch_factor_c<2>(p, njobs, s);
-}
-
 template <int CMAX>
 cudaError_t launch_cluster_t(const FactorParamsT<double> &p, const ClusterSlot *slots, int nclusters, int32_t *err,
                              cudaStream_t s) {
@@ -718,9 +700,7 @@ size_t cluster_smem_bytes(int n, int nc, size_t optin_per_block) {
 cudaError_t launch_factor_cluster(const FactorParamsT<double> &p, const ClusterSlot *slots, int nclusters,
                                   int32_t *err, cudaStream_t s) {
   if (nclusters <= 0) return cudaSuccess;
-  if (p.nc <= 16) return launch_cluster_t<1>(p, slots, nclusters, err, s);
-  if (p.nc <= 32) return launch_cluster_t<2>(p, slots, nclusters, err, s);
-  if (p.nc <= 64) return launch_cluster_t<4>(p, slots, nclusters, err, s);
+  if (p.n <= factor_fixed_max_rows(p.nc)) return launch_factor_fixed_cluster(p, slots, nclusters, s);
   return launch_cluster_t<8>(p, slots, nclusters, err, s);
 }
 
@@ -757,6 +737,8 @@ bool factor_tile_choice(int n, int nc, int leaf_h, size_t smem_per_sm, size_t re
   for (int c = max_cps < 3 ? max_cps : 3; c >= 1; --c) {
     int rows = factor_max_rows(nc, c, smem_per_sm, reserved_per_block, optin_per_block);
     if (rows > 512) rows = 512;  // the apply kernels stage at most 512 rows per tile
+    // the one-problem launches factor up to 64 columns in fixed point, on register tiles
+    if (max_cps >= 3 && factor_fixed_max_rows(nc) > 0) rows = std::min(rows, factor_fixed_max_rows(nc));
     // a third CTA per SM pays only while its tile still holds two triangles' worth of rows
     const int need = (c >= 3) ? 2 * n : n;
     if (rows >= need && rows >= 8) {
@@ -768,8 +750,14 @@ bool factor_tile_choice(int n, int nc, int leaf_h, size_t smem_per_sm, size_t re
   return false;
 }
 
-cudaError_t launch_factor(const FactorParamsT<double> &p, int njobs, cudaStream_t s, int ctas_per_sm) {
-  return launch_factor_any(p, njobs, ctas_per_sm, s);
+cudaError_t launch_factor(const FactorParamsT<double> &p, int njobs, int rows, cudaStream_t s, int ctas_per_sm) {
+  if (njobs <= 0) return cudaSuccess;
+  // up to 64 columns the fixed-point job is the faster one at every height (chains of 4M x 64
+  // 37 -> 19 ms, 16M x 16 9.6 -> 6.5 ms; a tree level of 64 columns 162 -> 97 us); above, its
+  // register tile would not hold a leaf in two CTAs per SM
+  if (rows <= factor_fixed_max_rows(p.nc)) return launch_factor_fixed(p, njobs, rows, s);
+  if (ctas_per_sm >= 3) return launch_factor_t<8, 3>(p, njobs, s);
+  return launch_factor_t<8, 2>(p, njobs, s);
 }
 
 cudaError_t launch_factor_batch(const BatchParams &p, int cmax, int grid, size_t smem_bytes, cudaStream_t s,

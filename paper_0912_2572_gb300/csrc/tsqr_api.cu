@@ -248,7 +248,7 @@ static void plan_clusters(Plan &pl, int64_t max_ctas) {
           int *pv = prod[t - b - 1];
           const int64_t l0 = 2 * il;  // local index of node 2i at level t - 1
           if (i < N[t - 1] / 2) {
-            sl[rank] = {pl.launches[t].job_begin + (int32_t)i, {pv[l0], pv[l0 + 1]}, 0};
+            sl[rank] = {pl.launches[t].job_begin + (int32_t)i, {pv[l0], pv[l0 + 1]}, t - b - 1};
             prod[t - b][il] = rank++;
           } else {
             prod[t - b][il] = pv[l0];  // passes up unchanged
@@ -562,7 +562,7 @@ static cudaError_t factor_launch(const tsqr_factors *F, FactorParams &p, int q, 
   const LaunchDesc &ld = pl.launches[q];
   p.job0 = ld.job_begin;
   ProfScope ps(q == 0 ? TSQR_PROF_FACTOR_CHAINS : TSQR_PROF_FACTOR_TREE, s);
-  return launch_factor(p, ld.job_count, s, q == 0 ? pl.ctas_per_sm : 2);
+  return launch_factor(p, ld.job_count, q == 0 ? pl.tile_h : pl.n, s, q == 0 ? pl.ctas_per_sm : 2);
 }
 
 // The binary tree levels (apply launches) that factorization launch q completes.

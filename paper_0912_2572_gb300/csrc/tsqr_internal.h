@@ -122,6 +122,8 @@ __device__ __forceinline__ double ld_state(const double *p) {
 #define TSQR_CHECK_OR_SKIP(cond, err)
 #endif
 
+struct ClusterSlot;
+
 template <typename R>
 struct FactorParamsT {
   const double *A;  // first-touch input for GEQRT/TSQRT tiles
@@ -158,7 +160,14 @@ size_t factor_smem_bytes(int nc, int ldt, size_t elem = sizeof(double));
 size_t f32wy_smem_extra_bytes();
 // ctas_per_sm: CTAs per SM the tile height was planned for (3 selects the build that fits
 // three in the register file; anything else, two).
-cudaError_t launch_factor(const FactorParamsT<double> &p, int njobs, cudaStream_t s, int ctas_per_sm = 2);
+// rows: the tallest tile of the launch's jobs.
+cudaError_t launch_factor(const FactorParamsT<double> &p, int njobs, int rows, cudaStream_t s, int ctas_per_sm = 2);
+// Fixed-point jobs (factor_fixed.cuh): the tallest tile at nc columns (0: not available), and
+// the launch of such a width.
+int factor_fixed_max_rows(int nc);
+cudaError_t launch_factor_fixed(const FactorParamsT<double> &p, int njobs, int rows, cudaStream_t s);
+cudaError_t launch_factor_fixed_cluster(const FactorParamsT<double> &p, const ClusterSlot *slots, int nclusters,
+                                        cudaStream_t s);
 int factor_max_rows(int nc, int ctas_per_sm, size_t smem_per_sm, size_t reserved_per_block,
                     size_t optin_per_block, size_t elem = sizeof(double));
 // Tile height and CTAs per SM of an FP64 factorization (nc columns, n of them A's, leaves
@@ -227,7 +236,7 @@ struct ClusterSlot {
   int32_t job;       // combine job of this CTA, or -1 (idle)
   int32_t child[2];  // cluster rank producing the pivot (0) / tile (1) triangle, or -1 when
                      // that triangle is complete in global memory (an earlier launch's)
-  int32_t pad;
+  int32_t round;     // the launch's level (0..2) this combine belongs to
 };
 // Shared memory of a cluster-tier combine CTA (the child's triangle, the dot products and
 // the pivot triangle), 0 when it exceeds the per-block maximum.

@@ -1,0 +1,119 @@
+"""The fixed-point factorization job (up to 64 columns): R, thin Q and the factorization
+itself at the edges of its tiles, of its number range and of its input checks, against the
+oracle. Tolerances are the library's stated ones (R 1e-12, backward error and orthogonality
+1e-13): the job carries 60 bits per column, more than FP64 arithmetic does."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_0912_2572_gb300 import inputs
+from conftest import to_dev, to_host
+
+pytestmark = pytest.mark.gpu
+
+
+def _rel(a, b):
+    return np.linalg.norm(a - b) / np.linalg.norm(b)
+
+
+def _check(ts, A, Ad=None, **kw):
+    F = ts.factor(to_dev(A) if Ad is None else Ad, **kw)
+    Q, R = to_host(F.form_q()), to_host(F.R)
+    F.free()
+    assert _rel(R, oracle.r_factor(A)) <= 1e-12
+    assert oracle.backward_error(A, Q, R) <= 1e-13
+    assert oracle.orth_error(Q) <= 1e-13
+    return R, Q
+
+
+# widths at the edges of the column groups (2, 4 and 8 columns a warp), heights at the edges
+# of a lane's rows and of the tile, chains whose last tile holds one row, tree nodes
+@pytest.mark.parametrize("m,n,h,arity,two", [
+    (1, 1, 1, 2, True), (513, 1, 512, 2, True), (1025, 8, 512, 2, True), (1537, 9, 512, 0, True),
+    (64, 16, 64, 2, False), (65, 16, 64, 2, True), (2049, 16, 256, 4, False), (577, 17, 288, 0, True),
+    (33, 32, 32, 2, False), (865, 32, 288, 0, True), (161, 33, 160, 2, True), (145, 64, 144, 0, True),
+    (433, 64, 144, 0, True), (64, 64, 64, 2, False), (4097, 63, 64, 3, False), (3000, 41, 41, 16, False),
+])
+def test_fixed_point_edges(cuda_lib, m, n, h, arity, two):
+    import paper_0912_2572_gb300 as ts
+    _check(ts, inputs.gaussian(m, n, m + n), leaf_h=h, arity=arity, two_level=two)
+
+
+@pytest.mark.parametrize("off", [0, 1])
+def test_fixed_point_misaligned_columns(cuda_lib, off):
+    """Odd leading dimensions and an 8-byte base: row pairs without 16-byte alignment."""
+    import torch
+    import paper_0912_2572_gb300 as ts
+    m, n, ld = 2000, 24, 2003
+    buf = torch.zeros(ld * n + 1, dtype=torch.float64, device="cuda")
+    Ad = buf[off:off + ld * n].view(n, ld).t()[:m]
+    A = inputs.gaussian(m, n, 5)
+    Ad.copy_(to_dev(A))
+    R0, Q0 = _check(ts, A)
+    R1, Q1 = _check(ts, A, Ad)
+    assert np.array_equal(R0, R1) and np.array_equal(Q0, Q1)
+
+
+def test_fixed_point_column_scales(cuda_lib):
+    """Columns scaled over 400 decades (each has its own exponent), and a chain whose tiles
+    grow by decades (the exponent grows along the chain)."""
+    import paper_0912_2572_gb300 as ts
+    m, n = 3000, 40
+    A = inputs.gaussian(m, n, 6)
+    s = 10.0 ** np.linspace(-100, 100, n)
+    F = ts.factor(to_dev(A * s), leaf_h=144, arity=0)
+    R, Q = to_host(F.R), to_host(F.form_q())
+    F.free()
+    assert _rel(R / s, oracle.r_factor(A)) <= 1e-12
+    assert oracle.orth_error(Q) <= 1e-13
+    g = 10.0 ** np.linspace(-8, 8, m)[:, None]
+    for B in (A * g, A * g[::-1]):
+        _check(ts, B, leaf_h=144, arity=0)
+
+
+def test_fixed_point_degenerate_columns(cuda_lib):
+    """Zero columns, a zero leading tile, repeated columns and a triangular matrix: H = I
+    where a tail is empty, R within the oracle's normwise error, Q orthonormal."""
+    import paper_0912_2572_gb300 as ts
+    m, n = 1200, 20
+    A = inputs.gaussian(m, n, 7)
+    A[:, 3] = 0.0
+    A[:, 9] = A[:, 2]
+    A[:300, 5] = 0.0
+    F = ts.factor(to_dev(A), leaf_h=100, arity=0)
+    R, Q = to_host(F.R), to_host(F.form_q())
+    F.free()
+    assert oracle.backward_error(A, Q, R) <= 1e-13 and oracle.orth_error(Q) <= 1e-13
+    assert np.all(R[:, 3] == 0.0) and abs(R[9, 9]) <= 1e-13 * np.linalg.norm(A[:, 9])
+    T = np.triu(inputs.gaussian(64, 64, 8))
+    F = ts.factor(to_dev(T), leaf_h=64)
+    # one rounding of each entry to 2^-61 of 2^E, where the column's norm is above 0.47 2^E
+    D = T * np.where(np.diag(T) < 0, -1.0, 1.0)[:, None]
+    assert np.all(np.abs(to_host(F.R) - D) <= 2.0 ** -59 * np.linalg.norm(T, axis=0))
+    F.free()
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf, 1e-290, 1e290])
+@pytest.mark.parametrize("row", [10, 500, 1990])
+def test_entries_outside_the_fixed_point_range(cuda_lib, bad, row):
+    """A tile with an entry the fixed-point form cannot take goes through the FP64 job, and
+    with it the rest of its chain: columns left of a non-finite entry are those of the clean
+    matrix, columns from it on are not finite; tiny entries behave as zeros to FP64 rounding
+    and huge ones (inside FP64, outside its squares) are not refused."""
+    import paper_0912_2572_gb300 as ts
+    m, n, c = 2000, 24, 7
+    A = inputs.gaussian(m, n, 9)
+    Rc = oracle.r_factor(A)
+    B = A.copy()
+    if bad == 1e-290:
+        B[row, :] = bad
+        F = ts.factor(to_dev(B), leaf_h=144, arity=0)
+        R, Q = to_host(F.R), to_host(F.form_q())
+        assert _rel(R, oracle.r_factor(B)) <= 1e-12 and oracle.orth_error(Q) <= 1e-13
+    else:
+        B[row, c] = bad
+        F = ts.factor(to_dev(B), leaf_h=144, arity=0)
+        R = to_host(F.R)
+        assert _rel(R[:, :c], Rc[:, :c]) <= 1e-12
+        assert not np.all(np.isfinite(R[:, c]))
+    F.free()
