@@ -41,6 +41,7 @@
 #include <cstdint>
 
 #include "factor_job.cuh"
+#include "fixed_point.cuh"
 
 namespace tsqr {
 namespace {
@@ -54,57 +55,6 @@ namespace {
 #else
 #define TSQR_CHECK_OR_SKIP_FX(cond, err, ret)
 #endif
-
-constexpr int kFxNone = -100000;     // no exponent yet (no nonzero entry seen)
-constexpr int kFxMaxExp = 900;       // entries of magnitude outside 2^+-900 (and non-finite ones)
-                                     // go through the FP64 job
-
-// a b + c. Written as the instruction: from (long long)a * b the compiler made full 64-bit
-// products wherever the operands were halves of 64-bit registers (four times the multiplies).
-__device__ __forceinline__ long long fx_mad(int a, int b, long long c) {
-  long long d;
-  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
-  return d;
-}
-
-// x 2^s, rounded to nearest for s < 0
-__device__ __forceinline__ long long fx_shift(long long x, int s) {
-  if (s >= 0) return s > 63 ? 0 : (long long)((unsigned long long)x << s);
-  if (s < -62) return 0;
-  return (x + (1ll << (-s - 1))) >> (-s);
-}
-
-__device__ __forceinline__ long long fx_of_double(long long bits, int sh) {  // round(x 2^sh)
-  const int e = (int)((bits >> 52) & 0x7ff);
-  if (e == 0 || e + sh <= 0) return 0;
-  return __double2ll_rn(__longlong_as_double(bits + ((long long)sh << 52)));
-}
-__device__ __forceinline__ double fx_to_double(long long x, int sh) {  // x 2^sh
-  const long long b = __double_as_longlong(__ll2double_rn(x));
-  return __longlong_as_double(x == 0 ? 0ll : b + ((long long)sh << 52));
-}
-
-// The magnitude bits of a double's high word, and its square relative to 2^(2t) as FP32
-// (20 mantissa bits), for the norm bound of a column whose largest exponent field is e (t =
-// e - 1022).
-__device__ __forceinline__ float fx_square_rel(unsigned habs, unsigned e) {
-  const int f = (int)(habs - ((e - 126u) << 20));
-  const float x = __int_as_float(f > 0 ? f << 3 : 0);
-  return x * x;
-}
-// Adds entries of squared norm sq 2^(2t) to a column of squared norm nb 2^(2E).
-__device__ __forceinline__ void fx_grow(int &E, float &nb, int t, float sq) {
-  const int base = max(E, t);
-  float s = sq * 1.00002f * exp2f((float)max(2 * (t - base), -140));
-  if (E > kFxNone) s += nb * exp2f((float)max(2 * (E - base), -140));
-  int b = base;
-  while (s >= 0.9f) {
-    ++b;
-    s *= 0.25f;
-  }
-  E = b;
-  nb = s;
-}
 
 // The scalars of reflector [alpha; x] from the raw column integers: alpha and T = alpha^2 +
 // ||x||^2 > 0. sh: the final shift of alpha and x;
@@ -154,18 +104,6 @@ __device__ __forceinline__ FxRefl fx_reflector(long long alpha, unsigned __int12
   f.y = yq >> 1;
   f.tq = (1ll << 59) + (long long)__umul64hi((unsigned long long)aa << 2, (unsigned long long)yq << 2);
   return f;
-}
-
-// ah 2^30 + al = a, al signed
-__device__ __forceinline__ void fx_limbs(long long a, int &h, int &l) {
-  h = (int)((a + (1ll << 29)) >> 30);
-  l = (int)((unsigned)a - ((unsigned)h << 30));
-}
-// a b / 2^S for S = 59 or 60, to within a unit
-template <int S>
-__device__ __forceinline__ long long fx_mul(int ah, int al, int2 b) {
-  const long long m = fx_mad(ah, b.y, fx_mad(al, b.x, 1ll << (S - 31)));
-  return fx_mad(ah, b.x, 0) * (1ll << (60 - S)) + (m >> (S - 30));
 }
 
 // Shared memory of the job: tails of two reflectors, the next pivot column, scalars (two

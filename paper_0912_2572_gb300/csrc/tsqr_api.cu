@@ -200,7 +200,6 @@ struct Plan {
   };
   std::vector<ClusterLaunch> cl_launches;
   std::vector<ClusterSlot> cl_slots;
-  std::vector<ApplyClusterSlot> cl_apply;  // the same slots seen top down (parents), for Q B
   int cl_base = 0;  // tree levels 1..cl_base run one launch each before the cluster launches
   // factorization launches (the chain launch, the per-level tree launches, the cluster launches)
   int factor_launches() const {
@@ -256,17 +255,6 @@ static void plan_clusters(Plan &pl, int64_t max_ctas) {
         }
       }
       pl.cl_slots.insert(pl.cl_slots.end(), sl, sl + kClusterSize);
-      // top down: each in-cluster child's parent and the side of the parent it continues
-      ApplyClusterSlot as[kClusterSize];
-      for (int r = 0; r < kClusterSize; ++r) as[r] = {sl[r].job, -1, 0, 0};
-      for (int r = 0; r < kClusterSize; ++r)
-        for (int q = 0; q < 2; ++q)
-          if (sl[r].job >= 0 && sl[r].child[q] >= 0) {
-            as[sl[r].child[q]].parent = r;
-            as[sl[r].child[q]].side = q;
-            as[r].kids |= 1 << q;
-          }
-      pl.cl_apply.insert(pl.cl_apply.end(), as, as + kClusterSize);
     }
     pl.cl_launches.push_back(cl);
   }
@@ -430,7 +418,6 @@ struct DevPlan {
   JobDesc *jobs = nullptr;
   TileDesc *tiles = nullptr;
   ClusterSlot *slots = nullptr;
-  ApplyClusterSlot *aslots = nullptr;
   int32_t *err = nullptr;  // the device error word
   ~DevPlan() {
     int cur = 0;
@@ -439,7 +426,6 @@ struct DevPlan {
     if (jobs) cudaFree(jobs);
     if (tiles) cudaFree(tiles);
     if (slots) cudaFree(slots);
-    if (aslots) cudaFree(aslots);
     cudaSetDevice(cur);
   }
 };
@@ -480,9 +466,6 @@ static tsqr_status get_plan(int64_t m, int n, int nc, int leaf_h, int arity, int
   if (!pl.cl_slots.empty()) {
     CUDA_TRY(cudaMalloc(&dp->slots, sizeof(ClusterSlot) * pl.cl_slots.size()));
     CUDA_TRY(cudaMemcpy(dp->slots, pl.cl_slots.data(), sizeof(ClusterSlot) * pl.cl_slots.size(),
-                        cudaMemcpyHostToDevice));
-    CUDA_TRY(cudaMalloc(&dp->aslots, sizeof(ApplyClusterSlot) * pl.cl_apply.size()));
-    CUDA_TRY(cudaMemcpy(dp->aslots, pl.cl_apply.data(), sizeof(ApplyClusterSlot) * pl.cl_apply.size(),
                         cudaMemcpyHostToDevice));
   }
   CUDA_TRY(device_error_word(&dp->err));
@@ -626,75 +609,34 @@ static tsqr_status apply_launch(const tsqr_factors *F, double *B, int64_t ldb, i
   // a tree level whose nodes, four CTAs each, still fit one wave of two CTAs per SM runs
   // 16 columns per CTA: each node's reflector steps get shorter
   const bool narrow = li > 0 && (int64_t)ld.job_count * 4 <= (int64_t)sms * 2;
+  if (kg > 8) {
+    CUDA_TRY(launch_apply_mma(p, ld.job_count, li == 0 ? pl.tile_h : pl.n, narrow ? 16 : 64, s));
+    return TSQR_OK;
+  }
   // one column over jobs of several tiles (the chains): tile pairs per warp
   const bool pairs = ld.job_count > 0 && pl.jobs[ld.job_begin].tile_count >= 2 && g_tile_pairs.load() != 0;
-  CUDA_TRY(launch_apply(p, ld.job_count, s, li == 0 ? pl.ctas_per_sm : 2, narrow ? 16 : 64, pairs));
+  CUDA_TRY(launch_apply(p, ld.job_count, s, pairs));
   return TSQR_OK;
 }
 
 // B is processed in groups of at most 64 columns (8 for the warp kernel path)
 static int apply_group(int k) { return (k <= 8) ? 8 : 64; }
 
-// The thin Q of up to 32 columns is formed in passes of 4 columns by the warp kernel: at
-// these widths the CTA kernel leaves most of its half-warps idle (reflector j touches
-// columns >= j only) between block barriers, and 4 columns per warp keep a job's staged
-// tile small enough for two or three CTAs of four jobs per SM.
-static int formq_group(int n) { return (n <= 32) ? 4 : 64; }
-
-// The cluster launch of F's plan that completes tree level li top down (the launch whose
-// highest level is li), for the columns [c0, c0 + kg) of B.
-static tsqr_status apply_cluster_launch(const tsqr_factors *F, double *B, int64_t ldb, int c0, int kg, int formq,
-                                        const Plan::ClusterLaunch &cl, cudaStream_t s) {
-  const Plan &pl = F->plan();
-  ApplyParams p{};
-  p.V = F->V;
-  p.ldv = F->ldv;
-  p.B = B;
-  p.ldb = ldb;
-  p.jobs = F->dp->jobs;
-  p.tiles = F->dp->tiles;
-  p.tau = F->tau;
-  p.scl = F->scl;
-  p.n = pl.n;
-  p.ldt = pl.n;
-  p.trans = 0;
-  p.formq = formq;
-  p.col0 = c0;
-  p.k = kg;
-  set_bounds(F, p);
-  ProfScope ps(formq ? TSQR_PROF_FORM_Q : TSQR_PROF_APPLY_Q, s);
-  CUDA_TRY(launch_apply_cluster(p, F->dp->aslots + cl.slot_begin, cl.nclusters, s));
-  return TSQR_OK;
-}
+// The thin Q of up to 8 columns is formed in passes of 4 columns by the warp kernel (one
+// panel of reflectors per tile would leave most of the tensor-core kernel's warps waiting
+// for it: 2^28 entries at n = 8 5.2 against 7.1 ms; at n = 16 9.7 against 7.2, n = 32 20.7
+// against 9.4), wider ones 64 columns at a time on the tensor cores.
+static int formq_group(int n) { return (n <= 8) ? 4 : 64; }
 
 static tsqr_status run_apply(const tsqr_factors *F, double *B, int64_t ldb, int k, int trans, int formq,
                              cudaStream_t s) {
   const Plan &pl = F->plan();
   const int nl = (int)pl.launches.size();
   const int group = formq ? formq_group(k) : apply_group(k);
-  // Q B top down with groups of more than 8 columns (the tile kernel's arithmetic, which the
-  // cluster launches share, so results stay bitwise those of the per-level launches): the
-  // levels of the cluster launches run as cluster launches, highest first
   for (int c0 = 0; c0 < k; c0 += group) {
     const int kg = std::min(group, k - c0);
-    const bool clustered = !trans && kg > 8 && !pl.cl_launches.empty() && F->dp->aslots;
     for (int q = 0; q < nl; ++q) {
-      const int li = trans ? q : nl - 1 - q;
-      tsqr_status st = TSQR_OK;
-      // a cluster launch runs only while all its CTAs (16 columns each) fit one wave at two
-      // per SM: on wider levels the pipelined launch is slower than the per-level launches
-      // (measured at 4M x 64: levels 3-5 of the thin Q 0.65 ms clustered, 0.43 ms per level)
-      const Plan::ClusterLaunch *hit = nullptr;
-      if (clustered && li > pl.cl_base)
-        for (const Plan::ClusterLaunch &cl : pl.cl_launches)
-          if (li >= cl.level_lo && li <= cl.level_hi) hit = &cl;
-      const int sms = device_info(F->device).sms;
-      if (hit && (int64_t)hit->nclusters * kClusterSize * ((kg + 15) / 16) > (int64_t)sms * 2) hit = nullptr;
-      if (hit) {
-        if (li == hit->level_hi) st = apply_cluster_launch(F, B, ldb, c0, kg, formq, *hit, s);
-      } else {
-        st = apply_launch(F, B, ldb, c0, kg, trans, formq, li, s);
-      }
+      tsqr_status st = apply_launch(F, B, ldb, c0, kg, trans, formq, trans ? q : nl - 1 - q, s);
       if (st != TSQR_OK) return st;
     }
   }

@@ -419,25 +419,15 @@ struct ApplyParamsT {
 
 using ApplyParams = ApplyParamsT<double>;
 
-// cols_per_cta caps the columns of B one CTA of the tile kernel handles (16, 32 or 64): a
-// launch with few jobs (a tree level) spreads a job's columns over more CTAs. Columns are
-// independent; only the summation order of a column's dot products changes with the cap.
-// tile_pairs: a launch whose jobs hold several tiles, with one column of B (Q^T b, Q b),
-// runs the tile-pair kernel (the job's tiles alternate between the two half-warps).
-cudaError_t launch_apply(const ApplyParamsT<double> &p, int njobs, cudaStream_t s, int ctas_per_sm = 2,
-                         int cols_per_cta = 64, bool tile_pairs = false);
+// Up to 8 columns of B. tile_pairs: a launch whose jobs hold several tiles, with one column of
+// B (Q^T b, Q b), runs the tile-pair kernel (the job's tiles alternate between the two
+// half-warps).
+cudaError_t launch_apply(const ApplyParamsT<double> &p, int njobs, cudaStream_t s, bool tile_pairs = false);
 
-// Cluster tier of B <- Q B (top down): one CTA per combine of a cluster launch of the
-// factorization's schedule, for 16 columns of B; parent = the cluster rank whose block this
-// node's pivot rows come from (-1: complete in global memory), side 0 = the parent's pivot
-// block, 1 = its tile block; kids bit q = the pivot (0) / tile (1) child is in the cluster.
-struct ApplyClusterSlot {
-  int32_t job;
-  int32_t parent, side, kids;
-};
-size_t apply_cluster_smem_bytes(int n);
-cudaError_t launch_apply_cluster(const ApplyParamsT<double> &p, const ApplyClusterSlot *slots, int nclusters,
-                                 cudaStream_t s);
+// More than 8 columns of B: on the tensor cores (apply_mma.cu). rows: the tallest tile of the
+// launch's jobs (at most 512). cols_per_cta caps the columns of B one CTA handles: a launch
+// with few jobs (a tree level) spreads a job's columns over more CTAs.
+cudaError_t launch_apply_mma(const ApplyParamsT<double> &p, int njobs, int rows, int cols_per_cta, cudaStream_t s);
 
 // ------------------------------------------------------------------- small kernels
 cudaError_t launch_extract_r(const double *V, int64_t ldv, int n, double *R, int64_t ldr,
