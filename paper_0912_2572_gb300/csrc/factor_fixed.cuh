@@ -16,7 +16,8 @@
 // update; the normwise error is the smaller one (Householder QR's bounds are normwise, per
 // column). The reflector's tail x and its pivot alpha are shifted left together until
 // 0.49 < ||[alpha; x]|| / 2^60 < 0.995 (exact: the shift is the only change), so a column
-// that cancelled down to few bits still gives a reflector orthogonal to 2^-58.
+// that cancelled down to few bits still gives a reflector orthogonal to 2^-58. Every few
+// columns what is left of a column is shifted up again (rescale below).
 //
 // Limbs. In the row loops a = ah 2^29 + al (C: al its low 29 bits; x and the coefficient q:
 // al signed), elsewhere 2^30; high limbs stay within 32 bits by the norm bounds. A product
@@ -34,9 +35,11 @@
 // on warp g or 11 - g, so each SM sub-partition holds an early and a late group.
 //
 // Measured on GB300 (chain launches, against the FP64 job): 4,194,304 x 64 in 144-row tiles
-// 37.0 -> 19.2 ms, 8M x 32 19.5 -> 11.0, 16M x 16 9.6 -> 6.0; a tree level of one 64-column
-// node 162 -> 95 us. A step of a 144 x 64 tile takes 4,800 cycles on one CTA and 6,500 on two:
-// the owner's dot products 1,650, coefficients 350, update 1,650, next reflector 1,700.
+// 37.0 -> 22.1 ms (18.9 without the rescaling and the unbiased scalars, with a 4 to 50 times
+// larger error of least-squares solutions at condition number 1e4), 16M x 16 9.6 -> 6.7; a
+// tree level of one 64-column node 162 -> 100 us. A step of a 144 x 64 tile takes 5,250 cycles
+// on one CTA and 6,850 on two: the owner's dot products 1,800, coefficients 570, update 1,700,
+// next reflector 2,000.
 #pragma once
 #include <cstdint>
 
@@ -58,14 +61,16 @@ namespace {
 
 // The scalars of reflector [alpha; x] from the raw column integers: alpha and T = alpha^2 +
 // ||x||^2 > 0. sh: the final shift of alpha and x;
-//   P = ||[alpha; x]|| 2^sh, D = |alpha| 2^sh + P, y = 2^118 / P, rD = 2^119 / D,
+//   P = ||[alpha; x]|| 2^sh, D = |alpha| 2^sh + P, y = 2^119 / P, rD = 2^119 / D,
 //   tq = 2^59 (1 + |alpha| / P)
 // The reciprocal square root and the reciprocal start from the FP32 functions (2^-20 or
 // better) and take one step of the third-order iterations
 //   y (1 + e/2 + 3/8 e^2), e = 1 - s y^2      and      r (1 + e + e^2), e = 1 - d r
 // (the binomial and geometric series cut after e^2: Householder's iterations of order three),
 // which leaves e^3 < 2^-60. On the FP64 pipe the same chain is a dozen dependent instructions
-// of 64 cycles.
+// of 64 cycles. A product cut to its upper half is taken at the middle of what it can be
+// (2 hi + 1): over a million rows the roundings of the entries average out, and errors of the
+// scalars with one sign (2^-59, from products cut down) were what remained of the error.
 struct FxRefl {
   long long P, y, rD, tq;
   int sh;
@@ -77,17 +82,19 @@ __device__ __forceinline__ FxRefl fx_reflector(long long alpha, unsigned __int12
   int k = L - 62;
   k += k & 1;
   const unsigned long long S = (unsigned long long)(k >= 0 ? T >> k : T << -k);  // [2^60, 2^62)
-  // s = S / 2^62 in [1/4, 1); P = 2^60 sqrt(s), or half of it where sqrt(s) is within 1% of 1
+  // s = S / 2^62 in [1/4, 1]; P = 2^60 sqrt(s), or half of it where sqrt(s) is within 1% of 1
   // (the high limb of a tail entry as large as P must stay below 2^31)
   const int ext = S >= 4519760000000000000ull ? 1 : 0;
   const float sf = __int2float_rn((int)(S >> 32)) * 0x1p-30f;
   const int y0 = __float2int_rn(rsqrtf(sf) * 0x1p29f);
-  const long long e = (1ll << 58) - (long long)__umul64hi(S, (unsigned long long)fx_mad(y0, y0, 0) << 2);
-  const int ee = (int)(e >> 12);
-  const long long u = (e >> 1) + ((3 * (fx_mad(ee, ee, 0) >> 34)) >> 3);
+  const unsigned long long y2 = (unsigned long long)fx_mad(y0, y0, 0) << 2;   // 2^60 y0^2
+  const long long e = (1ll << 59) - 1 - 2 * (long long)__umul64hi(S, y2);     // 2^59 (1 - s y0^2)
+  const int ee = (int)(e >> 13);
+  const long long u2e = e + ((3 * (fx_mad(ee, ee, 0) >> 33) + 2) >> 2);       // 2^59 (e + 3/4 e^2)
   const long long Y0 = (long long)y0 << 32;
-  const long long y = Y0 + (__mul64hi(Y0, u * (1ll << 24)) >> 18);  // 2^61 / sqrt(s)
-  f.P = (long long)(__umul64hi(S, (unsigned long long)y) << 1) >> ext;
+  const long long y = Y0 + ((__mul64hi(Y0, u2e * (1ll << 22)) + (1ll << 17)) >> 18);  // 2^61 / sqrt(s)
+  f.P = 2 * (long long)__umul64hi(S, (unsigned long long)y) + 1;
+  if (ext) f.P >>= 1;
   f.sh = 29 - (k >> 1) - ext;
   const long long af = fx_shift(alpha, f.sh);
   const long long aa = af < 0 ? -af : af;
@@ -95,21 +102,25 @@ __device__ __forceinline__ FxRefl fx_reflector(long long alpha, unsigned __int12
   const float df = __int2float_rn((int)(D >> 31)) * 0x1p-30f;
   const int r0 = __float2int_rn(__fdividef(1.0f, df) * 0x1p28f);
   const unsigned long long R0 = (unsigned long long)r0 << 32;
-  const long long e2 = (1ll << 58) - (long long)__umul64hi((unsigned long long)D << 1, R0);
-  const int ee2 = (int)(e2 >> 12);
-  const long long u2 = e2 + (fx_mad(ee2, ee2, 0) >> 34);
-  const long long r = (long long)R0 + (__mul64hi((long long)R0, u2 * (1ll << 23)) >> 17);  // 2^121 / D
+  const long long e2 = (1ll << 59) - 1 - 2 * (long long)__umul64hi((unsigned long long)D << 1, R0);  // 2^59 (1 - d r0)
+  const int ee2 = (int)(e2 >> 13);
+  const long long u2 = e2 + ((fx_mad(ee2, ee2, 0) + (1ll << 32)) >> 33);
+  const long long r = (long long)R0 + ((__mul64hi((long long)R0, u2 * (1ll << 22)) + (1ll << 16)) >> 17);  // 2^121 / D
   f.rD = (r + 2) >> 2;
-  const long long yq = ((y << ext) + 2) >> 2;  // 2^119 / P
-  f.y = yq >> 1;
-  f.tq = (1ll << 59) + (long long)__umul64hi((unsigned long long)aa << 2, (unsigned long long)yq << 2);
+  f.y = ((y << ext) + 2) >> 2;
+  f.tq = (1ll << 59) + (long long)((__umul64hi((unsigned long long)aa << 3, (unsigned long long)f.y << 2) + 1) >> 1);
   return f;
 }
 
+// Steps between two rescalings of a column.
 // Shared memory of the job: tails of two reflectors, the next pivot column, scalars (two
-// steps' limbs; every reflector's for the tile's end), column exponents and norms, R.
+// steps' limbs; every reflector's for the tile's end), column exponents and norms, R and the
+// scales of its row blocks.
+__host__ __device__ constexpr int fx_block(int n) { return n <= 8 ? 1 : n <= 16 ? 2 : n <= 32 ? 4 : 8; }
 __host__ __device__ constexpr size_t fx_smem_bytes(int n, int nc, int rows) {
-  return (size_t)3 * rows * 8 + 64 + (size_t)n * 24 + (size_t)((nc + 1) & ~1) * 8 + (size_t)n * (nc | 1) * 8;
+  const int rb = fx_block(n), nb = (n + rb - 1) / rb;
+  return (size_t)3 * rows * 8 + 64 + (size_t)n * 24 + (size_t)((nc + 1) & ~1) * 8 + (size_t)n * (nc | 1) * 8 +
+         (size_t)nb * ((nc + 1) & ~1) * 4;
 }
 
 // One job. Geometry: CPL columns per lane, LC lane columns, RPL (even) rows per lane; the
@@ -132,6 +143,9 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
   int *Es = ssh + 2 * n;
   float *nbs = reinterpret_cast<float *>(Es + ((nc + 1) & ~1));
   long long *Rs = reinterpret_cast<long long *>(nbs + ((nc + 1) & ~1));
+  const int rb = fx_block(n), rbl = 31 - __clz(rb), nbk = (n + rb - 1) >> rbl, lds = (nc + 1) & ~1;
+  int *Sc = reinterpret_cast<int *>(Rs + (size_t)n * ldr);  // Sc[b * lds + c]: R's rows of block b are
+                                                            // x 2^(60 - E_c + Sc)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int lr = lane % LR, lc = lane / LR;
   // SM sub-partition w mod 4 gets groups from both ends
@@ -139,6 +153,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
   const int cb = GC * grp;          // the group's first column
   const int64_t pr = job.piv_row;
   long long v[CPL][RPL];            // column cb + lc + LC t, rows 2 lr + 2 LR (r / 2) + r % 2
+  int cur[CPL];                     // and its scale: x 2^(60 - E_c + cur)
   TSQR_CHECK_OR_SKIP_FX(pr >= 0 && (p.rows == 0 || pr + n <= p.rows) && job.tile_begin >= 0 &&
                             (p.ntiles == 0 || job.tile_begin + job.tile_count <= p.ntiles) && nc <= NW * GC,
                         p.err, job.tile_count)
@@ -152,7 +167,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
       double *dst = gptr(pr, c);
       const int lim = c < n ? c + 1 : n;
       const int sh = exp_of(Es[c]) - 60;
-      for (int i = lane; i < lim; i += 32) dst[i] = fx_to_double(Rs[i * ldr + c], sh);
+      for (int i = lane; i < lim; i += 32) dst[i] = fx_to_double(Rs[i * ldr + c], sh - Sc[(i >> rbl) * lds + c]);
     }
   };
   auto row_of = [&](int r) { return 2 * lr + 2 * LR * (r >> 1) + (r & 1); };
@@ -166,7 +181,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
                               (p.nrefl == 0 || td.refl + n <= p.nrefl),
                           p.err, job.tile_count)
     const bool ge = (kind == GEQRT), tri = (kind == TTQRT);
-    const int j0 = tri ? off : 0;
+    const int j0 = tri ? (off >> rbl) << rbl : 0;  // reflectors before a piece's first row are H = I
     // the tile's bits; a child's triangle is zero below its diagonal
 #pragma unroll
     for (int t = 0; t < CPL; ++t) {
@@ -203,6 +218,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
         const double *src = gptr(pr, c);
         const int rl = c >= nc ? 0 : (c < n ? c + 1 : n);
         unsigned mx = 0;
+#pragma unroll 4
         for (int i = lr; i < rl; i += LR) mx = max(mx, (unsigned)__double2hiint(__ldcg(src + i)) & 0x7fffffffu);
 #pragma unroll
         for (int m = LR / 2; m >= 1; m >>= 1) mx = max(mx, __shfl_xor_sync(kFull, mx, m));
@@ -211,6 +227,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
         if (mx != 0 && !ok) bad = true;
         float s = 0.f;
         if (mx != 0 && ok)
+#pragma unroll 4
           for (int i = lr; i < rl; i += LR) s += fx_square_rel((unsigned)__double2hiint(__ldcg(src + i)) & 0x7fffffffu, e);
 #pragma unroll
         for (int m = LR / 2; m >= 1; m >>= 1) s += __shfl_xor_sync(kFull, s, m);
@@ -243,19 +260,26 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
     for (int t = 0; t < CPL; ++t) {
       const int c = cb + lc + LC * t;
       const int E = exp_of(En[t]);
-      if (c < nc) {
-        const int rl = c < n ? c + 1 : n;
-        if (tt == 0) {
-          if (!ge) {
-            const double *src = gptr(pr, c);
-            for (int i = lr; i < rl; i += LR)
-              Rs[i * ldr + c] = fx_of_double(__double_as_longlong(__ldcg(src + i)), 60 - E);
-          }
-        } else {
-          const int d = En[t] - Es[c];
-          if (d != 0)
-            for (int i = lr; i < rl; i += LR) Rs[i * ldr + c] = fx_shift(Rs[i * ldr + c], -d);
+      const int rl = c >= nc ? 0 : (c < n ? c + 1 : n);
+      if (tt == 0) {
+        // each block of R's rows at its own scale, its largest entry below 2^56
+        const double *src = gptr(pr, c);
+#pragma unroll 4
+        for (int k = 0; k < nbk; ++k) {
+          const int i = (k << rbl) + lr;
+          const bool in = !ge && lr < rb && i < rl;
+          const long long x = in ? __double_as_longlong(__ldcg(src + i)) : 0;
+          int e = (int)((x >> 52) & 0x7ff);
+#pragma unroll
+          for (int m = LR / 2; m >= 1; m >>= 1) e = max(e, __shfl_xor_sync(kFull, e, m));
+          const int sc = e == 0 ? 0 : min(max(E - (e - 1022) - 4, 0), 400);
+          if (in) Rs[i * ldr + c] = fx_of_double(x, 60 - E + sc);
+          if (lr == 0 && c < nc) Sc[k * lds + c] = sc;
         }
+      } else if (c < nc) {
+        const int d = En[t] - Es[c];  // the scales are relative to the exponent
+        if (d != 0 && Es[c] != kFxNone)
+          for (int k = lr; k < nbk; k += LR) Sc[k * lds + c] += d;
       }
       __syncwarp();  // the old exponent has been read
       if (c < nc && lr == 0) {
@@ -264,9 +288,76 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
       }
 #pragma unroll
       for (int r = 0; r < RPL; ++r) v[t][r] = fx_of_double(v[t][r], 60 - E);
+      cur[t] = 0;
     }
+    // what is left of the squared norm of a lane's column in the coefficient phase, in 4^E_c:
+    // R's finished rows are taken off (an upper bound up to rounding)
+    constexpr int kH = LR / 2;
+    const bool up = CPL == 2 && (lr & kH) != 0;
+    float qrem = up ? nbn[CPL - 1] : nbn[0];
     __syncthreads();
 
+    // Before reflector jn, every rb columns: a column that has become short of its 60 bits by
+    // two or more ([R's rows from jn on; tile]) is shifted up to fill them again. Columns
+    // lose most of their norm to the leading ones when they are nearly dependent; FP64 entries
+    // keep their bits then, and so do these. R's rows of the block take the column's scale.
+    // The estimate costs three instructions a step; the rescaling itself is rare on
+    // well-conditioned blocks (done at every block it took 15% of the chain's time).
+    auto rescale = [&](int jn) {
+      const int k = jn >> rbl;
+      // qrem 4^cur < 0.05
+      const bool mine = qrem < 0.05f * __int_as_float((127 - 2 * (up ? cur[CPL - 1] : cur[0])) << 23);
+      bool stay = !mine || cb + lc + (up ? LC : 0) < jn;
+#pragma unroll
+      for (int t = 0; t < CPL; ++t) {
+        const int c = cb + lc + LC * t;
+        stay = stay && (c < jn || c >= nc || Sc[k * lds + c] == cur[t]);
+      }
+      if (__all_sync(kFull, stay)) return;
+#pragma unroll
+      for (int t = 0; t < CPL; ++t) {
+        const int c = cb + lc + LC * t;
+        const bool on = c >= jn && c < nc;
+        const int rl = c < n ? c + 1 : n;
+        if (__any_sync(kFull, on && mine && up == (t == 1))) {
+          float q = 0.f;
+#pragma unroll
+          for (int r = 0; r < RPL; ++r) {
+            const float f = (!ge || row_of(r) >= jn) ? fabsf(__int2float_rn((int)(v[t][r] >> 32))) + 1.f : 0.f;
+            q = fmaf(f, f, q);
+          }
+          q *= exp2f((float)(-56 - 2 * cur[t]));
+          if (on && !ge)
+            for (int i = jn + lr; i < rl; i += LR) {
+              const float f = (fabsf(__int2float_rn((int)(Rs[i * ldr + c] >> 32))) + 1.f) *
+                              exp2f((float)(-28 - min(Sc[(i >> rbl) * lds + c], 90)));
+              q = fmaf(f, f, q);
+            }
+#pragma unroll
+          for (int m = LR / 2; m >= 1; m >>= 1) q += __shfl_xor_sync(kFull, q, m);
+          // the largest s with q 4^s < 0.9, at least the present one
+          int s2 = cur[t];
+          if (on) s2 = max(s2, min((126 - ((__float_as_int(q * 1.1112f) >> 23) & 0xff)) >> 1, 30));
+          const int d = s2 - cur[t];
+          if (on) {
+#pragma unroll
+            for (int r = 0; r < RPL; ++r) v[t][r] = (long long)((unsigned long long)v[t][r] << d);
+            cur[t] = s2;
+            if (up == (t == 1)) qrem = q;
+          }
+        }
+        if (on) {
+          const int d = cur[t] - Sc[k * lds + c];
+          if (!ge && d != 0 && lr < rb && jn + lr < rl) {
+            long long *x = Rs + (jn + lr) * ldr + c;
+            *x = fx_shift(*x, d);
+          }
+        }
+        __syncwarp();
+        if (on && lr == 0) Sc[k * lds + c] = cur[t];
+      }
+      __syncwarp();
+    };
     // reflector jn, published by the warp whose group holds column jn
     auto publish = [&](int jn) {
       const int b = jn & 1;
@@ -353,6 +444,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
         ssh[jn] = f.sh;
       }
     };
+    if (cb < nc && cb + GC > j0) rescale(j0);
     if (j0 >= cb && j0 < cb + GC) publish(j0);
     __syncthreads();
 
@@ -398,8 +490,6 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
         for (int t = 0; t < CPL; ++t) g[t] += m[t] >> 29;  // x C / 2^58
         // sum over the LR lanes of a column; with two columns per lane the first exchange
         // leaves the upper half of the lanes with the second one
-        constexpr int kH = LR / 2;
-        const bool up = CPL == 2 && (lr & kH) != 0;
         long long gt = g[0];
         if constexpr (CPL == 2) {
           const long long send = up ? g[0] : g[1];
@@ -410,13 +500,16 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
         const int c = cb + lc + (up ? LC : 0);
         const bool on = c > j && c < nc;
         const int2 rD = sb[4 * b], y = sb[4 * b + 1], tq = sb[4 * b + 2];
+        const float qsc = __int_as_float((99 - (up ? cur[CPL - 1] : cur[0])) << 23);  // 2^(-28 - cur)
         const long long p0 = on ? Rs[j * ldr + c] : 0;
         int h, l;
         fx_limbs((gt + 1) >> 1, h, l);
         const long long w = p0 + fx_mul<60>(h, l, rD);
         fx_limbs(w, h, l);
-        const long long nq = fx_mul<60>(h, l, y);
+        const long long nq = fx_mul<61>(h, l, y);
         const long long pk = p0 + fx_mul<59>(h, l, tq);
+        const float fk = __int2float_rn((int)(pk >> 32)) * qsc;
+        qrem = fmaf(-fk, fk, qrem);
         h = (int)((nq + (1ll << 28)) >> 29);  // -x's coefficient, / 2^58
         l = (int)((unsigned)nq - ((unsigned)h << 29));
         if (!on) h = l = 0;  // columns up to j are reflectors now
@@ -444,6 +537,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
               v[t][r + e] = fx_mad(xh[e], qh[t], v[t][r + e]) + (long long)(int)(z >> 29);
             }
         }
+        if (((j + 1) & (rb - 1)) == 0 && j + 1 < n) rescale(j + 1);
         if (j + 1 < n && j + 1 >= cb && j + 1 < cb + GC) publish(j + 1);
       }
       __syncthreads();
@@ -453,7 +547,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
     // them; identities for the rows a piece of a triangle does not reach
     for (int j = tid; j < n; j += 32 * NW) {
       p.tau[td.refl + j] = j < j0 ? 0.0 : fx_to_double(st[j], -59);
-      p.scl[td.refl + j] = j < j0 ? 0.0 : fx_to_double(sr[j], ssh[j] + 60 - exp_of(Es[j]) - 119);
+      p.scl[td.refl + j] = j < j0 ? 0.0 : fx_to_double(sr[j], ssh[j] + 60 - (exp_of(Es[j]) - Sc[(j >> rbl) * lds + j]) - 119);
     }
     // write the tile back: the leaf tile's reflectors below its diagonal (R goes out at the
     // chain's end), dense tails, or the child's triangle only
@@ -464,7 +558,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
       double *dst = gptr(r0, c);
       const int lim = tri && c < n ? min(ht, c + 1 - off) : ht;
       const int beg = ge ? (c < n ? c + 1 : n) : 0;
-      const int sh = exp_of(Es[c]) - 60;
+      const int sh = exp_of(Es[c]) - 60 - cur[t];
       const bool al = (reinterpret_cast<uintptr_t>(dst) & 15) == 0;
 #pragma unroll
       for (int r = 0; r < RPL; r += 2) {

@@ -201,11 +201,18 @@ __device__ __forceinline__ void bar_arrive_n(int id, int count) {
 // kernel, at its register cap, keeps that order). The row is not written before step j+1,
 // so both orders load the same values and give bitwise the same results.
 //
+// part: the CTA has more threads than the kThreads that run the job.
+//
 // COH: inputs and descriptors are read through L2 only (the resident kernel, whose inputs
 // and tables change while it runs); otherwise A goes through the read-only cache.
 template <int CMAX, bool EARLY_PF, bool COH = false>
-__device__ __forceinline__ void run_job(const FactorParamsT<double> &p, const JobDesc job, unsigned char *smraw) {
+__device__ __forceinline__ void run_job(const FactorParamsT<double> &p, const JobDesc job, unsigned char *smraw,
+                                        bool part = false) {
   using R = double;
+  auto sync = [part]() {
+    if (part) bar_sync_n(3, kThreads);
+    else __syncthreads();
+  };
   R *sm = reinterpret_cast<R *>(smraw);
   const int n = p.n, nc = p.nc, ldt = p.ldt;
   const int ncp = (nc + 7) & ~7;
@@ -256,7 +263,7 @@ __device__ __forceinline__ void run_job(const FactorParamsT<double> &p, const Jo
       p.tau[td.refl + j] = R(0);
       p.scl[td.refl + j] = R(0);
     }
-    __syncthreads();
+    sync();
 
     for (int j = j0; j < n; ++j) {
       int lo, hi;
@@ -336,7 +343,7 @@ __device__ __forceinline__ void run_job(const FactorParamsT<double> &p, const Jo
         }
         __syncwarp();
       }
-      __syncthreads();
+      sync();
     }
 
     // write the tile back: GEQRT -> R above / V below the diagonal, TSQRT -> dense
@@ -348,7 +355,7 @@ __device__ __forceinline__ void run_job(const FactorParamsT<double> &p, const Jo
       const int lim = (kind == TTQRT && c < n) ? max(0, min(ht, c + 1 - off)) : ht;
       warp_copy(dst, src, lim, lane, [](const double *q) { return *q; }, [](const double2 *q) { return *q; });
     }
-    __syncthreads();
+    sync();
   }
 }
 

@@ -63,11 +63,13 @@ __device__ __forceinline__ void fx_limbs(long long a, int &h, int &l) {
   h = (int)((a + (1ll << 29)) >> 30);
   l = (int)((unsigned)a - ((unsigned)h << 30));
 }
-// a b / 2^S for S = 59 or 60, to within a unit
+// a b / 2^S for S = 59, 60 or 61, to within a unit
 template <int S>
 __device__ __forceinline__ long long fx_mul(int ah, int al, int2 b) {
   const long long m = fx_mad(ah, b.y, fx_mad(al, b.x, 1ll << (S - 31)));
-  return fx_mad(ah, b.x, 0) * (1ll << (60 - S)) + (m >> (S - 30));
+  const long long h = fx_mad(ah, b.x, 0);
+  if constexpr (S <= 60) return h * (1ll << (60 - S)) + (m >> (S - 30));
+  else return (h + (m >> 30)) >> 1;
 }
 
 }  // namespace

@@ -195,7 +195,7 @@ extern "C" tsqr_status tsqr_lstsq_static(const double *A, int64_t m, int32_t n, 
   p.ldt = tile_h;
   for (int q = 0; q < nlaunches; ++q) {
     p.job0 = g_launches[q].job_begin;
-    STATIC_TRY(launch_factor(p, g_launches[q].job_count, q == 0 ? tile_h : n, s, q == 0 ? cps : 2));
+    STATIC_TRY(launch_factor(p, g_launches[q].job_count, q == 0 ? tile_h : n, s));
   }
   STATIC_TRY(launch_trsv(V, m, n, W, m, k, X, ldx, nullptr, status, s));
   int32_t hstatus = 0;

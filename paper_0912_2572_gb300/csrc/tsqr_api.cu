@@ -539,13 +539,12 @@ static cudaError_t factor_launch(const tsqr_factors *F, FactorParams &p, int q, 
     const Plan::ClusterLaunch &cl = pl.cl_launches[q - 1 - pl.cl_base];
     p.job0 = 0;
     ProfScope ps(TSQR_PROF_FACTOR_TREE, s);
-    return launch_factor_cluster(p, F->dp->slots + cl.slot_begin, cl.nclusters,
-                                 F->dp->err, s);
+    return launch_factor_cluster(p, F->dp->slots + cl.slot_begin, cl.nclusters, s);
   }
   const LaunchDesc &ld = pl.launches[q];
   p.job0 = ld.job_begin;
   ProfScope ps(q == 0 ? TSQR_PROF_FACTOR_CHAINS : TSQR_PROF_FACTOR_TREE, s);
-  return launch_factor(p, ld.job_count, q == 0 ? pl.tile_h : pl.n, s, q == 0 ? pl.ctas_per_sm : 2);
+  return launch_factor(p, ld.job_count, q == 0 ? pl.tile_h : pl.n, s);
 }
 
 // The binary tree levels (apply launches) that factorization launch q completes.
@@ -629,10 +628,10 @@ static int apply_group(int k) { return (k <= 8) ? 8 : 64; }
 static int formq_group(int n) { return (n <= 8) ? 4 : 64; }
 
 static tsqr_status run_apply(const tsqr_factors *F, double *B, int64_t ldb, int k, int trans, int formq,
-                             cudaStream_t s) {
+                             cudaStream_t s, int group = 0) {
   const Plan &pl = F->plan();
   const int nl = (int)pl.launches.size();
-  const int group = formq ? formq_group(k) : apply_group(k);
+  if (group == 0) group = formq ? formq_group(k) : apply_group(k);
   for (int c0 = 0; c0 < k; c0 += group) {
     const int kg = std::min(group, k - c0);
     for (int q = 0; q < nl; ++q) {
@@ -1907,7 +1906,10 @@ tsqr_status tsqr_lstsq(const double *A, int64_t m, int32_t n, int64_t lda, const
   f->stream = s;
   double *W = nullptr;  // Q^T B workspace (m-by-k)
   int32_t *status = nullptr;
-  const bool fused = (n + k) <= 128;
+  // B's columns are factored along unless they take A's over the edge of the eight-warp job
+  // (64 columns, two CTAs per SM; 1M x 64 with 4 right-hand sides 13.3 ms fused in sixteen
+  // warps): then Q^T B is a pass of its own
+  const bool fused = (n + k) <= 64 || (n > 64 && n + k <= 128);
   st = get_plan(m, n, fused ? n + k : n, leaf_h, arity, flags, f->dp);
   if (st == TSQR_OK) st = factors_alloc(f, s);
   if (st == TSQR_OK) {
@@ -1929,7 +1931,9 @@ tsqr_status tsqr_lstsq(const double *A, int64_t m, int32_t n, int64_t lda, const
       st = run_factor(f, A, lda, W, m, s);  // Q^T B computed with the factorization
     } else {
       st = run_factor(f, A, lda, nullptr, 0, s);
-      if (st == TSQR_OK) st = run_apply(f, W, m, k, 1, 0, s);
+      // eight columns at a time (FP64): the small components of Q^T B keep their bits, which
+      // an ill-conditioned R^{-1} magnifies
+      if (st == TSQR_OK) st = run_apply(f, W, m, k, 1, 0, s, 8);
     }
   }
   if (st == TSQR_OK) {

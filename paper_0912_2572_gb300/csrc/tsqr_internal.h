@@ -158,16 +158,10 @@ size_t factor_smem_bytes(int nc, int ldt, size_t elem = sizeof(double));
 // extra shared memory of an FP32 chain job with compact-WY panels (V twice, a chunk of
 // trailing columns, V^T C, T^T W, G and T)
 size_t f32wy_smem_extra_bytes();
-// ctas_per_sm: CTAs per SM the tile height was planned for (3 selects the build that fits
-// three in the register file; anything else, two).
-// rows: the tallest tile of the launch's jobs.
-cudaError_t launch_factor(const FactorParamsT<double> &p, int njobs, int rows, cudaStream_t s, int ctas_per_sm = 2);
-// Fixed-point jobs (factor_fixed.cuh): the tallest tile at nc columns (0: not available), and
-// the launch of such a width.
+// One-problem factorization launches (factor_fixed.cu), at most 128 columns. rows: the tallest
+// tile of the launch's jobs, at most factor_fixed_max_rows(nc).
 int factor_fixed_max_rows(int nc);
-cudaError_t launch_factor_fixed(const FactorParamsT<double> &p, int njobs, int rows, cudaStream_t s);
-cudaError_t launch_factor_fixed_cluster(const FactorParamsT<double> &p, const ClusterSlot *slots, int nclusters,
-                                        cudaStream_t s);
+cudaError_t launch_factor(const FactorParamsT<double> &p, int njobs, int rows, cudaStream_t s);
 int factor_max_rows(int nc, int ctas_per_sm, size_t smem_per_sm, size_t reserved_per_block,
                     size_t optin_per_block, size_t elem = sizeof(double));
 // Tile height and CTAs per SM of an FP64 factorization (nc columns, n of them A's, leaves
@@ -227,10 +221,8 @@ cudaError_t launch_factor_batch(const BatchParams &p, int cmax, int grid, size_t
 // ------------------------------------------------------- cluster tier of the tree
 // With TSQR_CLUSTER, three binary tree levels run in one launch of thread-block clusters
 // of kClusterSize CTAs: cluster c reduces the 8 consecutive triangles 8c..8c+7 of the
-// level below (4 + 2 + 1 combine jobs, one CTA each). A combine's column step j needs only
-// row j of each child's output triangle, which is final once the child has finished its
-// own step j, so the levels run as a pipeline: a parent waits for its children's progress
-// counters and reads their rows from their shared memory (distributed shared memory).
+// level below (4 + 2 + 1 combine jobs, one CTA each), a level per round between cluster
+// barriers.
 constexpr int kClusterSize = 8;
 struct ClusterSlot {
   int32_t job;       // combine job of this CTA, or -1 (idle)
@@ -241,9 +233,8 @@ struct ClusterSlot {
 // Shared memory of a cluster-tier combine CTA (the child's triangle, the dot products and
 // the pivot triangle), 0 when it exceeds the per-block maximum.
 size_t cluster_smem_bytes(int n, int nc, size_t optin_per_block);
-// err: the device error word (bit kErrTimeout set when a bounded wait gave up).
 cudaError_t launch_factor_cluster(const FactorParamsT<double> &p, const ClusterSlot *slots, int nclusters,
-                                  int32_t *err, cudaStream_t s);
+                                  cudaStream_t s);
 
 // Device error word: bit 1 (kErrTimeout) a bounded device wait gave up, bit 2 (kErrBounds)
 // an index check of a TSQR_CHECK build failed. One word per device.

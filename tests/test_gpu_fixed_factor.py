@@ -1,4 +1,4 @@
-"""The fixed-point factorization job (up to 64 columns): R, thin Q and the factorization
+"""The fixed-point factorization job: R, thin Q and the factorization
 itself at the edges of its tiles, of its number range and of its input checks, against the
 oracle. Tolerances are the library's stated ones (R 1e-12, backward error and orthogonality
 1e-13): the job carries 60 bits per column, more than FP64 arithmetic does."""
@@ -33,6 +33,7 @@ def _check(ts, A, Ad=None, **kw):
     (64, 16, 64, 2, False), (65, 16, 64, 2, True), (2049, 16, 256, 4, False), (577, 17, 288, 0, True),
     (33, 32, 32, 2, False), (865, 32, 288, 0, True), (161, 33, 160, 2, True), (145, 64, 144, 0, True),
     (433, 64, 144, 0, True), (64, 64, 64, 2, False), (4097, 63, 64, 3, False), (3000, 41, 41, 16, False),
+    (66, 65, 65, 2, True), (289, 127, 144, 0, True), (1153, 128, 144, 2, False), (900, 96, 100, 3, False),
 ])
 def test_fixed_point_edges(cuda_lib, m, n, h, arity, two):
     import paper_0912_2572_gb300 as ts
@@ -94,14 +95,14 @@ def test_fixed_point_degenerate_columns(cuda_lib):
 
 
 @pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf, 1e-290, 1e290])
-@pytest.mark.parametrize("row", [10, 500, 1990])
-def test_entries_outside_the_fixed_point_range(cuda_lib, bad, row):
+@pytest.mark.parametrize("row,n", [(10, 24), (500, 24), (1990, 24), (700, 90)])
+def test_entries_outside_the_fixed_point_range(cuda_lib, bad, row, n):
     """A tile with an entry the fixed-point form cannot take goes through the FP64 job, and
     with it the rest of its chain: columns left of a non-finite entry are those of the clean
     matrix, columns from it on are not finite; tiny entries behave as zeros to FP64 rounding
     and huge ones (inside FP64, outside its squares) are not refused."""
     import paper_0912_2572_gb300 as ts
-    m, n, c = 2000, 24, 7
+    m, c = 2000, 7
     A = inputs.gaussian(m, n, 9)
     Rc = oracle.r_factor(A)
     B = A.copy()
@@ -117,3 +118,22 @@ def test_entries_outside_the_fixed_point_range(cuda_lib, bad, row):
         assert _rel(R[:, :c], Rc[:, :c]) <= 1e-12
         assert not np.all(np.isfinite(R[:, c]))
     F.free()
+
+
+def test_non_finite_entry_in_a_wide_cluster_tree(cuda_lib):
+    """A combine of more than 64 columns in the cluster tier that meets a non-finite triangle
+    hands it to the FP64 job on half of its warps; the per-level tree gives the same R."""
+    import paper_0912_2572_gb300 as ts
+    m, n, c = 4000, 72, 30
+    A = inputs.gaussian(m, n, 10)
+    A[2500, c] = np.nan
+    R = {}
+    for cl in (False, True):
+        F = ts.factor(to_dev(A), leaf_h=144, two_level=False, cluster=cl)
+        R[cl] = to_host(F.R)
+        F.free()
+    assert np.array_equal(R[True], R[False], equal_nan=True)
+    A[2500, c] = 0.0
+    assert _rel(R[True][:, :c], oracle.r_factor(A)[:, :c]) <= 1e-12
+    # row i of R takes column c only at reflector i; reflector c spoils every row from c on
+    assert not np.any(np.isfinite(R[True][c, c:])) and not np.any(np.isfinite(R[True][:c, c]))
