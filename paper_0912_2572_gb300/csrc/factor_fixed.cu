@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) k_factor_fx_cluster(const Fa
 template <int CPL, int LC, int RPL, int NW = 8>
 cudaError_t launch_fx_cluster(FactorParamsT<double> p, const ClusterSlot *slots, int nclusters, cudaStream_t s) {
   p.ldt = p.n;  // the combines' tiles: what the shared memory below holds for the FP64 job
-  const size_t fx = fx_smem_bytes(p.n, p.nc, (32 / LC * RPL + 31) / 32 * 32), f64 = factor_smem_bytes(p.nc, p.ldt, sizeof(double));
+  const size_t fx = fx_smem_bytes(p.n, p.nc, LC, RPL), f64 = factor_smem_bytes(p.nc, p.ldt, sizeof(double));
   const size_t bytes = fx > f64 ? fx : f64;
   cudaError_t e = cudaFuncSetAttribute(k_factor_fx_cluster<CPL, LC, RPL, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)bytes);
@@ -72,7 +72,7 @@ cudaError_t launch_fx_cluster(FactorParamsT<double> p, const ClusterSlot *slots,
 
 template <int CPL, int LC, int RPL, int NW = 8>
 cudaError_t launch_fx(const FactorParamsT<double> &p, int njobs, cudaStream_t s) {
-  const size_t fx = fx_smem_bytes(p.n, p.nc, (32 / LC * RPL + 31) / 32 * 32), f64 = factor_smem_bytes(p.nc, p.ldt, sizeof(double));
+  const size_t fx = fx_smem_bytes(p.n, p.nc, LC, RPL), f64 = factor_smem_bytes(p.nc, p.ldt, sizeof(double));
   const size_t bytes = fx > f64 ? fx : f64;
   cudaError_t e = cudaFuncSetAttribute(k_factor_fx<CPL, LC, RPL, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;

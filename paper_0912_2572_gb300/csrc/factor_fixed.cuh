@@ -116,11 +116,14 @@ __device__ __forceinline__ FxRefl fx_reflector(long long alpha, unsigned __int12
 // Shared memory of the job: tails of two reflectors, the next pivot column, scalars (two
 // steps' limbs; every reflector's for the tile's end), column exponents and norms, R and the
 // scales of its row blocks.
-__host__ __device__ constexpr int fx_block(int n) { return n <= 8 ? 1 : n <= 16 ? 2 : n <= 32 ? 4 : 8; }
-__host__ __device__ constexpr size_t fx_smem_bytes(int n, int nc, int rows) {
-  const int rb = fx_block(n), nb = (n + rb - 1) / rb;
-  return (size_t)3 * rows * 8 + 64 + (size_t)n * 24 + (size_t)((nc + 1) & ~1) * 8 + (size_t)n * (nc | 1) * 8 +
-         (size_t)nb * ((nc + 1) & ~1) * 4;
+__host__ __device__ constexpr int fx_block(int n, int lr) {
+  const int rb = n <= 8 ? 1 : n <= 16 ? 2 : n <= 32 ? 4 : 8;
+  return rb < lr ? rb : lr;
+}
+__host__ __device__ constexpr size_t fx_smem_bytes(int n, int nc, int lc, int rpl) {
+  const int rb = fx_block(n, 32 / lc), nb = (n + rb - 1) / rb, rows = (32 / lc * rpl + 31) / 32 * 32;
+  return (size_t)3 * rows * 8 + 64 + (size_t)n * 24 + (size_t)((nc + 1) & ~1) * 12 +
+         ((size_t)n * nc - (size_t)n * (n - 1) / 2) * 8 + (size_t)nb * ((nc + 1) & ~1) * 2 + 16;
 }
 
 // One job. Geometry: CPL columns per lane, LC lane columns, RPL (even) rows per lane; the
@@ -128,12 +131,17 @@ __host__ __device__ constexpr size_t fx_smem_bytes(int n, int nc, int rows) {
 // nc <= NW GC. Returns the number of tiles done: all of them, or fewer when a tile holds an
 // entry the fixed-point form cannot take (not finite, or outside 2^+-900); the chain's state
 // is then in global memory, where the FP64 job goes on from.
-template <int CPL, int LC, int RPL, int NW, bool COH = false>
+//
+// KEEP = false (the batched kernels, which apply nothing later): only R and the right-hand
+// sides' pivot rows are written. A leaf tile is then a triangle-on-tile step from R = 0, so a
+// tile may be shorter than n, and all tiles are done: an entry that is not finite makes the R
+// it would have reached NaN.
+template <int CPL, int LC, int RPL, int NW, bool KEEP = true, bool COH = false>
 __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const JobDesc job, unsigned char *smraw) {
   constexpr int GC = CPL * LC, LR = 32 / LC, kRpw = (LR * RPL + 31) / 32, kRows = 32 * kRpw;
   static_assert(RPL % 2 == 0 && (CPL == 1 || CPL == 2), "row pairs; one or two columns");
   const int n = p.n, nc = p.nc;
-  const int ldr = nc | 1;
+  auto ro = [nc](int i) { return i * nc - i * (i + 1) / 2; };  // R(i, c), c >= i, at Rs[ro(i) + c]
   int2 *xb = reinterpret_cast<int2 *>(smraw);                       // tail limbs, buffer j mod 2
   long long *xw = reinterpret_cast<long long *>(xb + 2 * kRows);    // the next pivot column, raw
   int2 *sb = reinterpret_cast<int2 *>(xw + kRows);                  // limbs of rD, y, tq, buffer j mod 2
@@ -143,14 +151,15 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
   int *Es = ssh + 2 * n;
   float *nbs = reinterpret_cast<float *>(Es + ((nc + 1) & ~1));
   long long *Rs = reinterpret_cast<long long *>(nbs + ((nc + 1) & ~1));
-  const int rb = fx_block(n), rbl = 31 - __clz(rb), nbk = (n + rb - 1) >> rbl, lds = (nc + 1) & ~1;
-  int *Sc = reinterpret_cast<int *>(Rs + (size_t)n * ldr);  // Sc[b * lds + c]: R's rows of block b are
-                                                            // x 2^(60 - E_c + Sc)
+  const int rb = fx_block(n, LR), rbl = 31 - __clz(rb), nbk = (n + rb - 1) >> rbl, lds = (nc + 1) & ~1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int lr = lane % LR, lc = lane / LR;
   // SM sub-partition w mod 4 gets groups from both ends
   const int grp = (warp & 4) ? (warp & ~7) + 11 - (warp & 7) : warp;
   const int cb = GC * grp;          // the group's first column
+  int *cbad = reinterpret_cast<int *>(Rs + (size_t)n * nc - (size_t)n * (n - 1) / 2);  // KEEP = false: a
+                                      // column's first spoilt row (n: none)
+  short *Sc = reinterpret_cast<short *>(cbad + lds);  // R's rows of block b are x 2^(60 - E_c + Sc[b lds + c])
   const int64_t pr = job.piv_row;
   long long v[CPL][RPL];            // column cb + lc + LC t, rows 2 lr + 2 LR (r / 2) + r % 2
   int cur[CPL];                     // and its scale: x 2^(60 - E_c + cur)
@@ -163,11 +172,24 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
   auto exp_of = [](int E) { return E == kFxNone ? 0 : E; };  // nothing but zeros so far: any exponent
   // the chain's R to its pivot rows in global memory
   auto write_r = [&]() {
+    int first = n;  // the first spoilt column of A
+    if constexpr (!KEEP)
+      for (int c = n - 1; c >= 0; --c)
+        if (cbad[c] < n) first = c;
     for (int c = warp; c < nc; c += NW) {
       double *dst = gptr(pr, c);
       const int lim = c < n ? c + 1 : n;
       const int sh = exp_of(Es[c]) - 60;
-      for (int i = lane; i < lim; i += 32) dst[i] = fx_to_double(Rs[i * ldr + c], sh - Sc[(i >> rbl) * lds + c]);
+      for (int i = lane; i < lim; i += 32) {
+        const long long x = Rs[ro(i) + c];
+        const int s2 = sh - Sc[(i >> rbl) * lds + c];
+        double d;
+        if (KEEP || (s2 > -960 && s2 < 900)) d = fx_to_double(x, s2);
+        else d = scalbn(__ll2double_rn(x), s2);
+        if constexpr (!KEEP)
+          if (i >= cbad[c] || (c >= first && i >= first)) d = __longlong_as_double(0x7ff8000000000000ll);
+        dst[i] = d;
+      }
     }
   };
   auto row_of = [&](int r) { return 2 * lr + 2 * LR * (r >> 1) + (r & 1); };
@@ -180,7 +202,8 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
                               kind >= GEQRT && kind <= TTQRT && off >= 0 && off < n && td.refl >= 0 &&
                               (p.nrefl == 0 || td.refl + n <= p.nrefl),
                           p.err, job.tile_count)
-    const bool ge = (kind == GEQRT), tri = (kind == TTQRT);
+    const bool ge = KEEP && kind == GEQRT, tri = (kind == TTQRT);
+    const bool zero = tt == 0 && kind == GEQRT;  // nothing in R yet
     const int j0 = tri ? (off >> rbl) << rbl : 0;  // reflectors before a piece's first row are H = I
     // the tile's bits; a child's triangle is zero below its diagonal
 #pragma unroll
@@ -206,55 +229,87 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
       }
     }
     // exponents and norm bounds of the lane's columns
+    // rbad: the first of R's rows that an entry which is not finite spoils in the column
     bool bad = false;
-    int En[CPL];
+    int En[CPL], rbad[CPL];
     float nbn[CPL];
 #pragma unroll
     for (int t = 0; t < CPL; ++t) {
       const int c = cb + lc + LC * t;
       int E = (tt == 0 || c >= nc) ? kFxNone : Es[c];
       float nb = (tt == 0 || c >= nc) ? 0.f : nbs[c];
-      if (tt == 0 && !ge) {  // a tree node starts from the first child's triangle
-        const double *src = gptr(pr, c);
-        const int rl = c >= nc ? 0 : (c < n ? c + 1 : n);
-        unsigned mx = 0;
-#pragma unroll 4
-        for (int i = lr; i < rl; i += LR) mx = max(mx, (unsigned)__double2hiint(__ldcg(src + i)) & 0x7fffffffu);
+      rbad[t] = n;
+      // one set of entries: their largest exponent field, then their squares relative to it
+      auto grow = [&](unsigned mx, auto squares) {
 #pragma unroll
         for (int m = LR / 2; m >= 1; m >>= 1) mx = max(mx, __shfl_xor_sync(kFull, mx, m));
         const unsigned e = mx >> 20;
-        const bool ok = e >= 1023u - kFxMaxExp && e <= 1023u + kFxMaxExp;
-        if (mx != 0 && !ok) bad = true;
-        float s = 0.f;
-        if (mx != 0 && ok)
-#pragma unroll 4
-          for (int i = lr; i < rl; i += LR) s += fx_square_rel((unsigned)__double2hiint(__ldcg(src + i)) & 0x7fffffffu, e);
+        const bool ok = KEEP ? e >= 1023u - kFxMaxExp && e <= 1023u + kFxMaxExp : e != 0;
+        if (KEEP && mx != 0 && !ok) bad = true;
+        float s = ok ? squares(e) : 0.f;
 #pragma unroll
         for (int m = LR / 2; m >= 1; m >>= 1) s += __shfl_xor_sync(kFull, s, m);
-        if (mx != 0 && ok) fx_grow(E, nb, (int)e - 1022, s);
+        if (ok) fx_grow(E, nb, (int)e - 1022, s);
+      };
+      auto habs = [](long long x) { return (unsigned)(x >> 32) & 0x7fffffffu; };
+      if (tt == 0 && !zero && !ge) {  // a tree node starts from the first child's triangle
+        const double *src = gptr(pr, c);
+        const int rl = c >= nc ? 0 : (c < n ? c + 1 : n);
+        auto entry = [&](int i) {
+          const unsigned h = habs(__double_as_longlong(__ldcg(src + i)));
+          return !KEEP && h >= 0x7ff00000u ? 0u : h;
+        };
+        unsigned mx = 0;
+#pragma unroll 4
+        for (int i = lr; i < rl; i += LR) {
+          const unsigned h = habs(__double_as_longlong(__ldcg(src + i)));
+          if (!KEEP && h >= 0x7ff00000u) rbad[t] = min(rbad[t], i);
+          else mx = max(mx, h);
+        }
+        grow(mx, [&](unsigned e) {
+          float s = 0.f;
+#pragma unroll 4
+          for (int i = lr; i < rl; i += LR) s += fx_square_rel(entry(i), e);
+          return s;
+        });
       }
       unsigned mx = 0;
 #pragma unroll
-      for (int r = 0; r < RPL; ++r) mx = max(mx, (unsigned)(v[t][r] >> 32) & 0x7fffffffu);
+      for (int r = 0; r < RPL; ++r) {
+        const unsigned h = habs(v[t][r]);
+        if (!KEEP && h >= 0x7ff00000u) {
+          rbad[t] = tri ? min(rbad[t], off + row_of(r)) : 0;
+          v[t][r] = 0;
+        } else {
+          mx = max(mx, h);
+        }
+      }
+      grow(mx, [&](unsigned e) {
+        float s = 0.f;
 #pragma unroll
-      for (int m = LR / 2; m >= 1; m >>= 1) mx = max(mx, __shfl_xor_sync(kFull, mx, m));
-      const unsigned e = mx >> 20;
-      const bool ok = e >= 1023u - kFxMaxExp && e <= 1023u + kFxMaxExp;
-      if (mx != 0 && !ok) bad = true;
-      float s = 0.f;
+        for (int r = 0; r < RPL; ++r) s += fx_square_rel(habs(v[t][r]), e);
+        return s;
+      });
+      if constexpr (!KEEP)
 #pragma unroll
-      for (int r = 0; r < RPL; ++r) s += fx_square_rel((unsigned)(v[t][r] >> 32) & 0x7fffffffu, e);
-#pragma unroll
-      for (int m = LR / 2; m >= 1; m >>= 1) s += __shfl_xor_sync(kFull, s, m);
-      if (mx != 0 && ok) fx_grow(E, nb, (int)e - 1022, s);
+        for (int m = LR / 2; m >= 1; m >>= 1) rbad[t] = min(rbad[t], __shfl_xor_sync(kFull, rbad[t], m));
       En[t] = E;
       nbn[t] = nb;
     }
-    if (__syncthreads_or(bad)) {
-      if (tt > 0) write_r();
-      __threadfence();
+    if constexpr (KEEP) {
+      if (__syncthreads_or(bad)) {
+        if (tt > 0) write_r();
+        __threadfence();
+        __syncthreads();
+        return tt;
+      }
+    } else {
+#pragma unroll
+      for (int t = 0; t < CPL; ++t) {
+        const int c = cb + lc + LC * t;
+        if (lr == 0 && c < nc) cbad[c] = tt > 0 ? min(cbad[c], rbad[t]) : rbad[t];
+      }
       __syncthreads();
-      return tt;
     }
 #pragma unroll
     for (int t = 0; t < CPL; ++t) {
@@ -268,18 +323,19 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
         for (int k = 0; k < nbk; ++k) {
           const int i = (k << rbl) + lr;
           const bool in = !ge && lr < rb && i < rl;
-          const long long x = in ? __double_as_longlong(__ldcg(src + i)) : 0;
+          long long x = in && !zero ? __double_as_longlong(__ldcg(src + i)) : 0;
           int e = (int)((x >> 52) & 0x7ff);
+          if (!KEEP && e == 2047) x = e = 0;
 #pragma unroll
           for (int m = LR / 2; m >= 1; m >>= 1) e = max(e, __shfl_xor_sync(kFull, e, m));
           const int sc = e == 0 ? 0 : min(max(E - (e - 1022) - 4, 0), 400);
-          if (in) Rs[i * ldr + c] = fx_of_double(x, 60 - E + sc);
-          if (lr == 0 && c < nc) Sc[k * lds + c] = sc;
+          if (in) Rs[ro(i) + c] = fx_of_double(x, 60 - E + sc);
+          if (lr == 0 && c < nc) Sc[k * lds + c] = (short)sc;
         }
       } else if (c < nc) {
         const int d = En[t] - Es[c];  // the scales are relative to the exponent
         if (d != 0 && Es[c] != kFxNone)
-          for (int k = lr; k < nbk; k += LR) Sc[k * lds + c] += d;
+          for (int k = lr; k < nbk; k += LR) Sc[k * lds + c] = (short)(Sc[k * lds + c] + d);
       }
       __syncwarp();  // the old exponent has been read
       if (c < nc && lr == 0) {
@@ -329,7 +385,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
           q *= exp2f((float)(-56 - 2 * cur[t]));
           if (on && !ge)
             for (int i = jn + lr; i < rl; i += LR) {
-              const float f = (fabsf(__int2float_rn((int)(Rs[i * ldr + c] >> 32))) + 1.f) *
+              const float f = (fabsf(__int2float_rn((int)(Rs[ro(i) + c] >> 32))) + 1.f) *
                               exp2f((float)(-28 - min(Sc[(i >> rbl) * lds + c], 90)));
               q = fmaf(f, f, q);
             }
@@ -349,12 +405,12 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
         if (on) {
           const int d = cur[t] - Sc[k * lds + c];
           if (!ge && d != 0 && lr < rb && jn + lr < rl) {
-            long long *x = Rs + (jn + lr) * ldr + c;
+            long long *x = Rs + ro(jn + lr) + c;
             *x = fx_shift(*x, d);
           }
         }
         __syncwarp();
-        if (on && lr == 0) Sc[k * lds + c] = cur[t];
+        if (on && lr == 0) Sc[k * lds + c] = (short)cur[t];
       }
       __syncwarp();
     };
@@ -368,7 +424,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
           for (int r = 0; r < RPL; r += 2)
             *reinterpret_cast<longlong2 *>(xw + row_of(r)) = make_longlong2(v[t][r], v[t][r + 1]);
       __syncwarp();
-      const long long alpha = ge ? xw[jn] : Rs[jn * ldr + jn];
+      const long long alpha = ge ? xw[jn] : Rs[ro(jn) + jn];
       long long x[kRpw];
       long long hh = 0, hl = 0, ll = 0;
       unsigned any = 0;
@@ -390,7 +446,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
         for (int r = 0; r < kRpw; ++r) xb[b * kRows + lane + 32 * r] = make_int2(0, 0);
         if (lane < 3) sb[4 * b + lane] = make_int2(0, 0);
         if (lane == 0) {
-          Rs[jn * ldr + jn] = alpha;
+          Rs[ro(jn) + jn] = alpha;
           sr[jn] = 0;
           st[jn] = 0;
           ssh[jn] = 0;
@@ -438,7 +494,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
         sb[4 * b] = a;
         sb[4 * b + 1] = c;
         sb[4 * b + 2] = d;
-        Rs[jn * ldr + jn] = fx_shift(neg ? f.P : -f.P, -f.sh);
+        Rs[ro(jn) + jn] = fx_shift(neg ? f.P : -f.P, -f.sh);
         sr[jn] = rD;
         st[jn] = f.tq;
         ssh[jn] = f.sh;
@@ -464,7 +520,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
 #pragma unroll
               for (int r = 1; r < kPr; ++r)
                 if (r == rj) z = v[t][r];
-              if (c > j && c < nc) Rs[j * ldr + c] = z;
+              if (c > j && c < nc) Rs[ro(j) + c] = z;
             }
           __syncwarp();
         }
@@ -501,7 +557,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
         const bool on = c > j && c < nc;
         const int2 rD = sb[4 * b], y = sb[4 * b + 1], tq = sb[4 * b + 2];
         const float qsc = __int_as_float((99 - (up ? cur[CPL - 1] : cur[0])) << 23);  // 2^(-28 - cur)
-        const long long p0 = on ? Rs[j * ldr + c] : 0;
+        const long long p0 = on ? Rs[ro(j) + c] : 0;
         int h, l;
         fx_limbs((gt + 1) >> 1, h, l);
         const long long w = p0 + fx_mul<60>(h, l, rD);
@@ -514,7 +570,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
         l = (int)((unsigned)nq - ((unsigned)h << 29));
         if (!on) h = l = 0;  // columns up to j are reflectors now
         __syncwarp();        // every lane of a column has read p0
-        if (on && (CPL == 2 ? lr % kH : lr) == 0) Rs[j * ldr + c] = pk;
+        if (on && (CPL == 2 ? lr % kH : lr) == 0) Rs[ro(j) + c] = pk;
         int qh[CPL], ql[CPL];
         qh[0] = h;
         ql[0] = l;
@@ -543,6 +599,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
       __syncthreads();
     }
 
+    if constexpr (!KEEP) continue;
     // the reflectors' scalars: v = [1; scale x], H = I - tau v v^T, as the apply kernels read
     // them; identities for the rows a piece of a triangle does not reach
     for (int j = tid; j < n; j += 32 * NW) {

@@ -20,7 +20,7 @@
 // loses nothing: entries not yet claimed stay in the rings for the next launch.
 #include <cstdint>
 
-#include "factor_job.cuh"
+#include "batch_job.cuh"
 #include "refine_task.cuh"
 #include "tsqr_internal.h"
 
@@ -209,12 +209,9 @@ __device__ void run_chain(const ResParams &p, int slot, int jb, unsigned char *s
       fp.B = in.B;
       fp.ldb = in.ldb;
       fp.tiles = it.tiles;
-      fp.tau = chain ? static_cast<double *>(in.tau) : in.tau64;
-      fp.scl = chain ? static_cast<double *>(in.scl) : in.scl64;
       fp.n = in.n;
       fp.nc = in.n + in.k;
-      fp.ldt = chain ? in.ldt : in.ldt_tree;
-      run_job<kResCmax, false, true>(fp, jd, smraw);
+      run_batch_job<kResCmax, true, true>(fp, jd, smraw, !chain);
     }
     if (bj.parent < 0) {
       __threadfence();

@@ -348,8 +348,8 @@ static int split_tree_tiles(Plan &pl, int h) {
 // Chooses the tile height and CTAs per SM of the factor kernel for nc columns: two
 // resident CTAs when the tile still holds at least n rows (one CTA's scalar phase is
 // then hidden behind the other's updates), otherwise one.
-// max_cps: the persistent batched kernel is built for two CTAs per SM; the one-problem
-// launches may run three.
+// max_cps: the persistent batched kernel is built for two CTAs per SM and has tiles of its
+// own; the one-problem launches may run three.
 static bool choose_tiles(const DeviceInfo &di, int n, int nc, int leaf_h, int &tile_h, int &cps,
                          size_t elem = sizeof(double), int max_cps = 3) {
   if (elem == sizeof(float)) {  // register-tile FP32 chains: fixed 128-row tiles
@@ -357,6 +357,11 @@ static bool choose_tiles(const DeviceInfo &di, int n, int nc, int leaf_h, int &t
     tile_h = std::min(kF32TileRows, std::max(leaf_h, n));
     cps = 2;
     return true;
+  }
+  if (max_cps == 2) {
+    tile_h = batch_job_rows(nc);
+    cps = 2;
+    return nc <= 144;
   }
   return factor_tile_choice(n, nc, leaf_h, di.smem_sm, di.reserved, di.optin, max_cps, tile_h, cps);
 }
@@ -702,7 +707,7 @@ struct BatchBuild {
   int32_t count = 0;
   std::vector<tsqr_batch_item> items;
   std::vector<Plan> plans;
-  std::vector<int32_t> prec, tree_rows, wy;
+  std::vector<int32_t> prec, wy;
   bool wy_any = false;
   size_t smem = 0;
   int cmax = 1, grid = 0;
@@ -751,7 +756,6 @@ tsqr_status batch_build_on(DeviceInfo di, const tsqr_batch_item *items, int32_t 
   b.items.assign(items, items + count);
   b.plans.resize(count);
   b.prec.resize(count);
-  b.tree_rows.resize(count);
   b.wy.assign(count, 0);
   const int32_t wy_min = g_wy_min_n.load();
   int cps_min = 2;
@@ -768,16 +772,21 @@ tsqr_status batch_build_on(DeviceInfo di, const tsqr_batch_item *items, int32_t 
     int th = 0, cps = 0;
     if (!choose_tiles(di, it.n, nc, 1 << 20, th, cps, elem, 2))
       return fail(TSQR_ERR_UNSUPPORTED, "item %d: no tile fits shared memory", q);
-    const int64_t tiles = (it.m + th - 1) / th;
+    // chain_tiles counts tiles of the height that two CTAs per SM hold in shared memory as
+    // doubles, whatever the job's own tiles
+    int tc = th, cps64 = 0;
+    if (!mixed && !factor_tile_choice(it.n, nc, 1 << 20, di.smem_sm, di.reserved, di.optin, 2, tc, cps64)) tc = th;
+    const int64_t tiles = (it.m + tc - 1) / tc;
     // mixed items: FP32 chains kMixedChainFactor times longer (fewer FP64 tree combines)
     const int64_t Lq = mixed ? (int64_t)L * kMixedChainFactor : L;
+    // a chain's triangle takes the place of its first n rows: leaves of at least n rows
+    const int leaf = th * ((it.n + th - 1) / th);
     const int64_t G = std::max<int64_t>(1, (tiles + Lq / 2) / Lq);
-    tsqr_status st = make_plan_on(di, b.plans[q], it.m, it.n, nc, th, arity, TSQR_TWO_LEVEL, mixed, G, 2);
+    tsqr_status st = make_plan_on(di, b.plans[q], it.m, it.n, nc, leaf, arity, TSQR_TWO_LEVEL, mixed, G, 2);
     if (st != TSQR_OK) return st;
-    // tree nodes (FP64) in pieces that fit the chains' CTAs per SM
-    const int node_rows = b.tree_rows[q] = split_tree_tiles(
-        b.plans[q], factor_max_rows(nc, b.plans[q].ctas_per_sm, di.smem_sm, di.reserved, di.optin, sizeof(double)));
-    size_t chain_smem = factor_smem_bytes(nc, b.plans[q].tile_h, elem);
+    // tree nodes (FP64) in pieces that fit the job's register tile
+    split_tree_tiles(b.plans[q], nc <= 64 ? it.n : batch_job_rows(nc));
+    size_t chain_smem = mixed ? factor_smem_bytes(nc, b.plans[q].tile_h, elem) : 0;
     if (mixed && wy_min > 0 && it.n >= wy_min && it.n > 16) {
       // compact-WY FP32 chains, if their buffers still fit two CTAs per SM
       const size_t wsm = chain_smem + f32wy_smem_extra_bytes();
@@ -788,11 +797,12 @@ tsqr_status batch_build_on(DeviceInfo di, const tsqr_batch_item *items, int32_t 
       }
     }
     b.smem = std::max(b.smem, chain_smem);
-    b.smem = std::max(b.smem, factor_smem_bytes(nc, node_rows, sizeof(double)));
+    b.smem = std::max(b.smem, batch_job_smem(it.n, nc));
     b.smem = std::max(b.smem, sizeof(double) * (size_t)it.n * std::max(it.k, 1));
     while (16 * b.cmax < nc) b.cmax *= 2;
     cps_min = std::min(cps_min, b.plans[q].ctas_per_sm);
   }
+  if (2 * (b.smem + di.reserved + kBatchSmemSlack) > di.smem_sm) cps_min = 1;
   // ctas_per_sm = 1 leaves room on every SM for a CTA of another stream's kernel (the
   // server overlaps one batch's refinement with the next batch's factorization)
   b.grid = di.sms * (ctas_per_sm > 0 ? std::min(cps_min, (int)ctas_per_sm) : cps_min);
@@ -989,7 +999,6 @@ void batch_bind(BatchBuild &b, char *base) {
     bi.k = pl.mixed ? 0 : it.k;
     bi.B = bi.k > 0 ? (double *)(base + o.B) : nullptr;
     bi.ldt = pl.tile_h;
-    bi.ldt_tree = b.tree_rows[q];
     bi.mixed = pl.mixed ? 1 : 0;
     bi.wy = b.wy[q];
   }
@@ -1049,7 +1058,8 @@ tsqr_status batch_enqueue(const BatchBuild &b, char *base, cudaStream_t s, bool 
   bp.nchains = b.nchains;
   {
     ProfScope ps(profile ? TSQR_PROF_BATCH : -1, s);
-    CUDA_TRY(launch_factor_batch(bp, b.cmax, b.grid, b.smem, s, b.wy_any));
+    const bool fp64_items = std::find(b.prec.begin(), b.prec.end(), (int32_t)TSQR_FP64) != b.prec.end();
+    CUDA_TRY(launch_factor_batch(bp, b.cmax, b.grid, b.smem, s, fp64_items, b.wy_any));
   }
   if (!b.rinst.empty()) {
     RefineParams rp{};
@@ -1199,8 +1209,11 @@ tsqr_status tsqr::resident_plan(const tsqr_batch_item &it, int32_t chain_tiles, 
   for (int32_t q = 0; q < b->count; ++q) {
     const int nc = b->plans[q].mixed ? it.n : it.n + it.k;
     const size_t elem = b->plans[q].mixed ? sizeof(float) : sizeof(double);
-    smem = std::max(smem, factor_smem_bytes(nc, b->plans[q].tile_h, elem));
-    smem = std::max(smem, factor_smem_bytes(nc, b->tree_rows[q], sizeof(double)));
+    if (b->plans[q].mixed) smem = std::max(smem, factor_smem_bytes(nc, b->plans[q].tile_h, elem));
+    smem = std::max(smem, batch_job_smem(it.n, nc));
+    // FP64 requests whose n rows of doubles do not fit two CTAs per SM are admitted at one
+    // only (they need less since the job keeps its tile in registers; the rule is kept)
+    if (!b->plans[q].mixed) smem = std::max(smem, factor_smem_bytes(nc, it.n, sizeof(double)));
     smem = std::max(smem, sizeof(double) * (size_t)it.n * std::max(it.k, 1));
   }
   out.smem = std::max(smem, b->rsmem);

@@ -193,7 +193,6 @@ struct BatchInst {
   int64_t ldx;
   int32_t *status;  // device flag set to 4 when R is singular (solve only)
   int32_t n, k, ldt, mixed;
-  int32_t ldt_tree;  // shared-memory rows of a tree-node tile (a piece of a triangle)
   int32_t wy;        // mixed items: FP32 chains by compact-WY panels with 3xTF32 tensor-core
                      // updates (run_job_f32wy) instead of the unblocked register tile
 };
@@ -215,8 +214,14 @@ struct BatchParams {
   int32_t nchains;
 };
 
+// Shared memory and tallest tile of an FP64 job of the batched kernels (nc columns, n of them
+// the matrix's); a tile may be shorter than n.
+size_t batch_job_smem(int n, int nc);
+int batch_job_rows(int nc);
+cudaError_t launch_factor_batch_wide(const BatchParams &p, int grid, size_t smem_bytes, cudaStream_t s,
+                                     bool fp64_items, bool wy);
 cudaError_t launch_factor_batch(const BatchParams &p, int cmax, int grid, size_t smem_bytes, cudaStream_t s,
-                                bool wy = false);
+                                bool fp64_items, bool wy = false);
 
 // ------------------------------------------------------- cluster tier of the tree
 // With TSQR_CLUSTER, three binary tree levels run in one launch of thread-block clusters

@@ -268,3 +268,53 @@ def test_batch_of_ten_thousand_sampled_against_oracle(cuda_lib):
         assert rel(R, oracle.r_factor(A)) <= (1e-12 if q % 2 == 0 else 1e-5), f"item {q}"
     del buf, items, outs
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("n,k", [(8, 0), (16, 2), (17, 0), (32, 3), (33, 0), (60, 4), (64, 1), (100, 8), (128, 0), (128, 16)])
+def test_fp64_items_at_the_edges_of_their_tiles(cuda_lib, n, k):
+    """Heights around n, around one and two of the job's tiles (512, 288, 144, 72 and 36 rows by
+    width) and several chains, against the oracle and the one-problem path: tiles shorter than
+    n, leaves of several tiles, tree nodes in pieces, an odd leading dimension."""
+    import torch
+    import paper_0912_2572_gb300 as ts
+    nc = n + k
+    th = 512 if nc <= 16 else 288 if nc <= 32 else 144 if nc <= 64 else 72 if nc <= 128 else 36
+    items, host = [], []
+    for q, m in enumerate((n, n + 1, th, th + 1, 2 * th + n, 40 * th + 7)):
+        m = max(m, n)
+        A, B = inputs.gaussian(m, n, 50 + q), inputs.gaussian(m, max(k, 1), 60 + q)
+        buf = torch.zeros((n, m + 1), dtype=torch.float64, device="cuda")
+        Ad = buf.t()[:m]
+        Ad.copy_(to_dev(A))
+        host.append((A, B))
+        items.append({"A": Ad, "prec": ts.FP64, **({"B": to_dev(B)} if k else {})})
+    outs, st = ts.batch_solve(items, chain_tiles=4, status=True)
+    assert st == [0] * len(items)
+    for (A, B), (R, X) in zip(host, outs):
+        Ro = oracle.r_factor(A)
+        assert np.linalg.norm(to_host(R) - Ro) <= 1e-12 * np.linalg.norm(Ro)
+        if k and A.shape[0] >= 2 * n:  # square problems are as ill-conditioned as their A
+            Xo = oracle.lstsq(A, B)
+            assert np.linalg.norm(to_host(X) - Xo) <= 1e-11 * np.linalg.norm(Xo)
+
+
+def test_fp64_items_with_entries_that_are_not_finite(cuda_lib):
+    """R of an item with a NaN in column c: column c is NaN, columns before it are those of the
+    clean matrix, rows from c on are NaN, through chains, pieces of nodes and levels, as in the
+    one-problem factorization; other items of the batch are untouched. Entries near the edge of
+    the supported range are taken."""
+    import paper_0912_2572_gb300 as ts
+    for n, c in ((20, 7), (100, 40)):
+        A = inputs.gaussian(6000, n, 70 + n)
+        Ab = A.copy()
+        Ab[4321, c] = np.nan
+        (Rb, _), (Rc, _), (Rh, _) = ts.batch_solve([{"A": to_dev(Ab)}, {"A": to_dev(A)}, {"A": to_dev(A * 1e140)}])
+        Rb, Rc, Rh = to_host(Rb), to_host(Rc), to_host(Rh)
+        Ro = oracle.r_factor(A)
+        assert np.linalg.norm(Rc - Ro) <= 1e-12 * np.linalg.norm(Ro)
+        assert np.linalg.norm(Rh / 1e140 - Ro) <= 1e-12 * np.linalg.norm(Ro)
+        up = np.triu(np.ones((n, n), bool))
+        bad = up & ((np.arange(n)[None, :] == c) | ((np.arange(n)[:, None] >= c) & (np.arange(n)[None, :] >= c)))
+        assert np.all(np.isnan(Rb[bad]))
+        good = up & ~bad & (np.arange(n)[None, :] < c)
+        assert np.linalg.norm((Rb - Ro)[good]) <= 1e-12 * np.linalg.norm(Ro)
