@@ -6,8 +6,9 @@
 // applies jobs launch by launch, tiles and reflectors in factorization order; Q applies
 // everything in reverse.
 //
-// B with at most 8 columns runs here, and the thin Q of up to 8 columns in passes of 4; more
-// columns go to the tensor-core kernel (apply_mma.cu). k_apply_warp: one warp per job; each
+// B with at most 8 columns runs here, and the thin Q of up to 8 columns in passes of 4, and 9
+// to 16 columns against few reflectors (k_apply_tile); other widths go to the tensor-core
+// kernel (apply_mma.cu). k_apply_warp: one warp per job; each
 // reflector is a dot product over the tile rows, one warp-level transpose-reduce, and an
 // update; no block barrier is needed. With 4 columns a job stages 16.6 KB of a 512-row tile,
 // so three CTAs of four jobs fit per SM, and the independent jobs of a sub-partition's three
@@ -394,6 +395,137 @@ __global__ void __launch_bounds__(128, 3) k_apply_vec(const ApplyParamsT<double>
   for (int j = lane; j < n; j += 32) B[pr + j] = Pf[j];
 }
 
+// ------------------------------------------- 9..16 columns, few reflectors: a CTA per job
+// With few reflectors per tile the tensor-core kernel is bound by what it does once per tile
+// and panel (digits of V and of the tile, eight of its warps on two column groups); here the
+// tile of up to 16 columns is in shared memory, a half-warp per column, and the next
+// reflector's tail and pivot row are loaded one step ahead. The columns rotate over the
+// warps with the reflector, so that no SM sub-partition's FP64 pipe takes the extra half-warp
+// of an odd count at every step. Q^T B, n rows cleared and Q B of 1,000,000 x 8 with 9 / 16
+// columns 1.35 / 1.78 ms (1.99 / 2.02 on the tensor cores, 2 x 1.88 in passes of 8 columns),
+// x 12 with 16 2.52 (2.79), x 16 with 9 2.41 (2.75).
+constexpr int kTileThreads = 256, kTileCols = 16;
+
+template <int RM, int MINB>
+__global__ void __launch_bounds__(kTileThreads, MINB) k_apply_tile(const ApplyParamsT<double> p) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int n = p.n, ldt = p.ldt, kc = p.k;
+  double *Bt = reinterpret_cast<double *>(smraw);  // kTileCols columns of ldt rows
+  double *PC = Bt + (size_t)kTileCols * ldt;       // dot products, then update coefficients
+  double *PV = PC + kTileCols;                     // the pivot row (TSQRT / TTQRT)
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, hl = tid & 15;
+  TSQR_CHECK_OR_SKIP(p.njobs == 0 || p.job0 + (int)blockIdx.x < p.njobs, p.err)
+  const JobDesc job = p.jobs[p.job0 + blockIdx.x];
+  const int64_t pr = job.piv_row;
+  auto bp = [&](int64_t row, int c) -> double * { return p.B + row + (int64_t)(p.col0 + c) * p.ldb; };
+  TSQR_CHECK_OR_SKIP(kc <= kTileCols && pr >= 0 && (p.rows == 0 || pr + n <= p.rows) &&
+                         (p.ntiles == 0 || job.tile_begin + job.tile_count <= p.ntiles),
+                     p.err)
+  const int nt = job.tile_count;
+  for (int q = 0; q < nt; ++q) {
+    const TileDesc td = p.tiles[job.tile_begin + (p.trans ? q : nt - 1 - q)];
+    const int ht = td.nrows, kind = td.kind;
+    const bool ge = (kind == GEQRT);
+    const int64_t r0 = td.row0;
+    TSQR_CHECK_OR_SKIP(r0 >= 0 && ht >= 1 && ht <= ldt && (p.rows == 0 || r0 + ht <= p.rows) && td.refl >= 0 &&
+                           (p.nrefl == 0 || td.refl + n <= p.nrefl),
+                       p.err)
+    const double *Vt = p.V + r0;
+    for (int c = warp; c < kc; c += kTileThreads / 32)
+      for (int i = lane; i < ht; i += 32) Bt[(size_t)c * ldt + i] = *bp(r0 + i, c);
+    const int j0 = p.trans ? 0 : n - 1;
+    if (!ge && tid < kc) PV[tid] = __ldcg(bp(pr + j0, tid));
+    double xv[RM], xn[RM];
+    double tau = 0.0, sc = 0.0, tau_n = 0.0, sc_n = 0.0;  // warp 0's
+    if (warp == 0) {
+      tau = __ldg(p.tau + td.refl + j0);
+      sc = __ldg(p.scl + td.refl + j0);
+    }
+    auto load = [&](double(&x)[RM], int j) {
+      int lo, hi;
+      refl_rows(kind, j, ht, lo, hi, td.off);
+#pragma unroll
+      for (int r = 0; r < RM; ++r) {
+        const int i = lo + hl + 16 * r;
+        x[r] = (i < hi) ? __ldg(Vt + i + (int64_t)j * p.ldv) : 0.0;
+      }
+    };
+    load(xv, j0);
+    __syncthreads();
+    for (int s = 0; s < n; ++s) {
+      const int j = p.trans ? s : n - 1 - s, jn = p.trans ? j + 1 : j - 1;
+      const bool more = s + 1 < n;
+      int lo, hi;
+      refl_rows(kind, j, ht, lo, hi, td.off);
+      double pf = 0.0;
+      const bool do_pf = !ge && warp == 1 && more && lane < kc;
+      if (more) {
+        if (warp == 0) {
+          tau_n = __ldg(p.tau + td.refl + jn);
+          sc_n = __ldg(p.scl + td.refl + jn);
+        }
+        load(xn, jn);
+        if (do_pf) pf = __ldcg(bp(pr + jn, lane));
+      }
+      const int rw = (warp + s) & 7;        // this reflector's pair of columns
+      const int c = 2 * rw + ((tid >> 4) & 1);
+      double *b = Bt + (size_t)c * ldt;
+      const int ra = (hi - lo + 15) >> 4;
+      if (2 * rw < kc) {  // warp-uniform
+        double acc = 0.0;
+#define TSQR_TDOT(r)                                                                        \
+  {                                                                                         \
+    const int i = lo + hl + 16 * (r);                                                       \
+    if (i < hi && c < kc) acc = fma(xv[r], b[i], acc);                                      \
+  }
+        TSQR_ROW_SLOTS(ra, RM, TSQR_TDOT)
+#undef TSQR_TDOT
+#pragma unroll
+        for (int m = 8; m >= 1; m >>= 1) acc += __shfl_xor_sync(kFull, acc, m);
+        if (hl == 0 && c < kc) PC[c] = acc;
+      }
+      __syncthreads();
+      if (warp == 0 && lane < kc) {
+        const double piv = ge ? Bt[(size_t)lane * ldt + j] : PV[lane];
+        const double w = fma(sc, PC[lane], piv);
+        const double np = fma(-tau, w, piv);
+        PC[lane] = tau * sc * w;
+        if (ge) Bt[(size_t)lane * ldt + j] = np;
+        else *bp(pr + j, lane) = np;
+      }
+      __syncthreads();
+      if (2 * rw < kc) {
+        const double cf = c < kc ? PC[c] : 0.0;
+#define TSQR_TUPD(r)                                                                        \
+  {                                                                                         \
+    const int i = lo + hl + 16 * (r);                                                       \
+    if (i < hi && c < kc) b[i] = fma(-cf, xv[r], b[i]);                                     \
+  }
+        TSQR_ROW_SLOTS(ra, RM, TSQR_TUPD)
+#undef TSQR_TUPD
+      }
+      if (do_pf) PV[lane] = pf;
+#pragma unroll
+      for (int r = 0; r < RM; ++r) xv[r] = xn[r];
+      tau = tau_n;
+      sc = sc_n;
+      __syncthreads();
+    }
+    for (int c = warp; c < kc; c += kTileThreads / 32)
+      for (int i = lane; i < ht; i += 32) *bp(r0 + i, c) = Bt[(size_t)c * ldt + i];
+    __syncthreads();
+  }
+}
+
+template <int RM, int MINB>
+cudaError_t launch_tile_t(const ApplyParamsT<double> &p, int njobs, cudaStream_t s) {
+  const size_t bytes = sizeof(double) * ((size_t)kTileCols * p.ldt + 2 * kTileCols);
+  cudaError_t e = cudaFuncSetAttribute(k_apply_tile<RM, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e != cudaSuccess) return e;
+  k_apply_tile<RM, MINB><<<njobs, kTileThreads, bytes, s>>>(p);
+  return cudaGetLastError();
+}
+
 template <int K, int RW, typename R>
 cudaError_t launch_warp_t(const ApplyParamsT<R> &p, int njobs, cudaStream_t s) {
   const size_t bytes = sizeof(R) * 4 * ((size_t)p.ldt + p.n) * K;
@@ -452,6 +584,14 @@ cudaError_t launch_apply(const ApplyParamsT<double> &p, int njobs, cudaStream_t 
     return cudaErrorInvalidValue;
   }
   return launch_apply_any(p, njobs, s);
+}
+
+cudaError_t launch_apply_tile(const ApplyParamsT<double> &p, int njobs, cudaStream_t s) {
+  if (njobs <= 0 || p.k <= 0) return cudaSuccess;
+  if (p.k > kTileCols || p.formq || p.ldt > 512) return cudaErrorInvalidValue;
+  if (p.ldt <= 128) return launch_tile_t<8, 2>(p, njobs, s);
+  if (p.ldt <= 256) return launch_tile_t<16, 2>(p, njobs, s);
+  return launch_tile_t<32, 1>(p, njobs, s);
 }
 
 }  // namespace tsqr

@@ -7,8 +7,10 @@
 namespace tsqr {
 namespace {
 
-// CMAX: the widest item of the launch, in 16 columns. A group per warp: 2, 4, 8, 16 or 32
-// columns of up to 36 entries a lane; nodes up to 64 columns wide take builds of their own
+// CMAX: the widest item of the launch, in 16 columns. A group per warp: 2, 4, 8, 12, 16 or 24
+// columns of up to 36 entries a lane (42 above 128 columns: 56-row tiles; 36-row tiles of 32
+// columns a warp took 32 served FP64 requests 76.8 ms, these and the 96-row tiles of 12 columns
+// a warp for 65..96 columns 69.4); nodes up to 64 columns wide take builds of their own
 // height (a 512-row tile's registers would all be walked for 16 rows). CHAINS: the launch has
 // FP64 items; without their builds the kernel's other jobs compile better (16.7M x 32 mixed:
 // the factorization 10.4 ms, 11.5 beside them).
@@ -29,10 +31,12 @@ __device__ __forceinline__ void run_batch_job(const FactorParamsT<double> &p, co
       if (node) run_job_fx<2, 4, 8, NW, false, COH>(p, job, smraw);
       else if constexpr (CHAINS) run_job_fx<2, 4, 18, NW, false, COH>(p, job, smraw);
     }
+  } else if (p.nc <= 96) {
+    if constexpr (CMAX >= 8) run_job_fx<3, 4, 12, NW, false, COH>(p, job, smraw);
   } else if (p.nc <= 128) {
     if constexpr (CMAX >= 8) run_job_fx<2, 8, 18, NW, false, COH>(p, job, smraw);
   } else {
-    if constexpr (CMAX >= 16 && CHAINS) run_job_fx<2, 16, 18, NW, false, COH>(p, job, smraw);
+    if constexpr (CMAX >= 16 && CHAINS) run_job_fx<3, 8, 14, NW, false, COH>(p, job, smraw);
   }
 }
 

@@ -1,29 +1,7 @@
-// TSQR factorization kernels (sm_103a), FP64 and FP32 instantiations. The job code they
-// share with the resident kernel is in factor_job.cuh; the notes below describe it.
-//
-// One CTA runs one job (a chain of tiles sharing n pivot rows, see tsqr_internal.h).
-// Each tile is staged in shared memory and factored column by column with Householder
-// reflections (paper §2.2); the pivot row of reflector j is the tile's own row j (GEQRT,
-// a leaf) or row j of the job's running triangle R held in global memory (TSQRT: the
-// flat-tree step [R; tile], TTQRT: the tree combine [R; R_child], paper §2.3).
-//
-// GB300 design notes. FP64 runs on a narrow pipe (2 DFMA/clk/SM: each of the four SM
-// sub-partitions takes one FP64 warp instruction per 64 cycles) and a warp instruction
-// costs the same with masked lanes, so the kernel keeps warps full, spends FP64 issue
-// slots only on the factorization itself, and spreads them evenly over sub-partitions:
-//   * per column step j the dot products p_k = sum_i b_ij b_ik (k > j) are one Gram-row
-//     pass, so one reduction per step;
-//   * a worker half-warp owns columns; each lane walks 1/16 of the rows, so a value is
-//     reduced over only 16 lanes, by a transpose-reduce that spends about one DADD per
-//     value instead of four;
-//   * reflectors are stored unscaled with (tau, scale) beside them, so the update of a
-//     trailing element is exactly one DFMA: b_ik -= (tau*scale*w_k) * b_ij;
-//   * every warp issues exactly as many column slots as it owns at each step: a
-//     predicated-off DFMA still occupies the FP64 pipe, so the column guards are
-//     warp-uniform branches, not predicates;
-//   * the reflector's scalar chain runs on its own warp, overlapped with the dot
-//     products (run_job below), and the column dealing rotates with the step so that no
-//     sub-partition's FP64 pipe carries more than its share.
+// The batched persistent kernel up to 64 columns (sm_103a; factor_wide.cu has the wider
+// builds) and the sizes of the factorization jobs. The jobs themselves are in batch_job.cuh
+// (FP64 items and tree nodes in 64-bit fixed point, factor_fixed.cuh; FP32 chains of mixed
+// items, factor_job.cuh); the one-problem launches are in factor_fixed.cu.
 #include <algorithm>
 #include <cstdint>
 #include <type_traits>
@@ -115,9 +93,12 @@ size_t batch_job_smem(int n, int nc) {
   if (nc <= 16) return fx_smem_bytes(n, nc, 1, 16);
   if (nc <= 32) return fx_smem_bytes(n, nc, 2, 18);
   if (nc <= 64) return fx_smem_bytes(n, nc, 4, 18);
-  return nc <= 128 ? fx_smem_bytes(n, nc, 8, 18) : fx_smem_bytes(n, nc, 16, 18);
+  if (nc <= 96) return fx_smem_bytes(n, nc, 4, 12);
+  return nc <= 128 ? fx_smem_bytes(n, nc, 8, 18) : fx_smem_bytes(n, nc, 8, 14);
 }
 
-int batch_job_rows(int nc) { return nc <= 16 ? 512 : nc <= 32 ? 288 : nc <= 64 ? 144 : nc <= 128 ? 72 : 36; }
+int batch_job_rows(int nc) {
+  return nc <= 64 ? factor_fixed_max_rows(nc) : nc <= 96 ? 96 : nc <= 128 ? 72 : 56;
+}
 
 }  // namespace tsqr

@@ -70,6 +70,25 @@ cudaError_t launch_fx_cluster(FactorParamsT<double> p, const ClusterSlot *slots,
   return cudaLaunchKernelEx(&cfg, k_factor_fx_cluster<CPL, LC, RPL, NW>, p, slots);
 }
 
+// Chains of up to 4 and of 9 to 12 columns stay on the FP64 job (half-warps of the CTA own a
+// column each): in fixed point such a tile has too few columns for its conversions (2 and 4:
+// thin QR of 1.5M rows in 128-row tiles 0.42 and 0.78 ms, 0.53 and 0.91 in fixed point), or
+// leaves half of each group empty (1.5M x 12 in 256-row leaves 3.10, 3.31). So do tree nodes of
+// up to 8 rows with 9 to 16 columns (200,000 x 8 with one right-hand side 0.43 ms, 0.46). Four
+// CTAs per SM fit at 64 registers.
+__global__ void __launch_bounds__(kThreads, 4) k_factor_narrow(const FactorParamsT<double> p) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  run_job<1, true>(p, p.jobs[p.job0 + blockIdx.x], smraw);
+}
+
+cudaError_t launch_narrow(const FactorParamsT<double> &p, int njobs, cudaStream_t s) {
+  const size_t bytes = factor_smem_bytes(p.nc, p.ldt, sizeof(double));
+  cudaError_t e = cudaFuncSetAttribute(k_factor_narrow, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e != cudaSuccess) return e;
+  k_factor_narrow<<<njobs, kThreads, bytes, s>>>(p);
+  return cudaGetLastError();
+}
+
 template <int CPL, int LC, int RPL, int NW = 8>
 cudaError_t launch_fx(const FactorParamsT<double> &p, int njobs, cudaStream_t s) {
   const size_t fx = fx_smem_bytes(p.n, p.nc, LC, RPL), f64 = factor_smem_bytes(p.nc, p.ldt, sizeof(double));
@@ -87,6 +106,8 @@ int factor_fixed_max_rows(int nc) { return nc <= 16 ? 512 : nc <= 32 ? 288 : nc 
 cudaError_t launch_factor(const FactorParamsT<double> &p, int njobs, int rows, cudaStream_t s) {
   if (njobs <= 0) return cudaSuccess;
   if (p.nc > 128 || rows > factor_fixed_max_rows(p.nc)) return cudaErrorInvalidValue;
+  const bool narrow = rows > 64 ? p.nc <= 4 || (p.nc >= 9 && p.nc <= 12) : p.n <= 8 && p.nc >= 9 && p.nc <= 16;
+  if (narrow) return launch_narrow(p, njobs, s);
   if (p.nc <= 8) {
     if (rows <= 64) return launch_fx<1, 1, 2>(p, njobs, s);
     if (rows <= 256) return launch_fx<1, 1, 8>(p, njobs, s);

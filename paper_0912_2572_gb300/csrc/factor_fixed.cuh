@@ -139,7 +139,7 @@ __host__ __device__ constexpr size_t fx_smem_bytes(int n, int nc, int lc, int rp
 template <int CPL, int LC, int RPL, int NW, bool KEEP = true, bool COH = false>
 __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const JobDesc job, unsigned char *smraw) {
   constexpr int GC = CPL * LC, LR = 32 / LC, kRpw = (LR * RPL + 31) / 32, kRows = 32 * kRpw;
-  static_assert(RPL % 2 == 0 && (CPL == 1 || CPL == 2), "row pairs; one or two columns");
+  static_assert(RPL % 2 == 0 && CPL >= 1 && CPL <= 3 && LR >= 4, "row pairs; one to three columns");
   const int n = p.n, nc = p.nc;
   auto ro = [nc](int i) { return i * nc - i * (i + 1) / 2; };  // R(i, c), c >= i, at Rs[ro(i) + c]
   int2 *xb = reinterpret_cast<int2 *>(smraw);                       // tail limbs, buffer j mod 2
@@ -290,9 +290,10 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
         for (int r = 0; r < RPL; ++r) s += fx_square_rel(habs(v[t][r]), e);
         return s;
       });
-      if constexpr (!KEEP)
+      if constexpr (!KEEP) {
 #pragma unroll
         for (int m = LR / 2; m >= 1; m >>= 1) rbad[t] = min(rbad[t], __shfl_xor_sync(kFull, rbad[t], m));
+      }
       En[t] = E;
       nbn[t] = nb;
     }
@@ -348,9 +349,18 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
     }
     // what is left of the squared norm of a lane's column in the coefficient phase, in 4^E_c:
     // R's finished rows are taken off (an upper bound up to rounding)
-    constexpr int kH = LR / 2;
-    const bool up = CPL == 2 && (lr & kH) != 0;
-    float qrem = up ? nbn[CPL - 1] : nbn[0];
+    constexpr int kH = LR / 2, kQ = LR / 4;
+    // the column of the coefficient phase: one per half of a column's lanes, or per quarter of
+    // them (three columns, the last quarter idle)
+    const int sel = CPL == 1 ? 0 : CPL == 2 ? (lr & kH) / kH : lr / kQ;
+    const bool up = (lr & kH) != 0;
+    auto pick = [sel](const auto (&a)[CPL]) {
+      if constexpr (CPL == 1) return a[0];
+      else if constexpr (CPL == 2) return sel ? a[1] : a[0];
+      else return sel == 0 ? a[0] : sel == 1 ? a[1] : a[2];
+    };
+    const int cs = sel < CPL ? cb + lc + LC * sel : nc;
+    float qrem = pick(nbn);
     __syncthreads();
 
     // Before reflector jn, every rb columns: a column that has become short of its 60 bits by
@@ -362,8 +372,8 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
     auto rescale = [&](int jn) {
       const int k = jn >> rbl;
       // qrem 4^cur < 0.05
-      const bool mine = qrem < 0.05f * __int_as_float((127 - 2 * (up ? cur[CPL - 1] : cur[0])) << 23);
-      bool stay = !mine || cb + lc + (up ? LC : 0) < jn;
+      const bool mine = qrem < 0.05f * __int_as_float((127 - 2 * pick(cur)) << 23);
+      bool stay = !mine || cs < jn || cs >= nc;
 #pragma unroll
       for (int t = 0; t < CPL; ++t) {
         const int c = cb + lc + LC * t;
@@ -375,7 +385,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
         const int c = cb + lc + LC * t;
         const bool on = c >= jn && c < nc;
         const int rl = c < n ? c + 1 : n;
-        if (__any_sync(kFull, on && mine && up == (t == 1))) {
+        if (__any_sync(kFull, on && mine && sel == t)) {
           float q = 0.f;
 #pragma unroll
           for (int r = 0; r < RPL; ++r) {
@@ -399,7 +409,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
 #pragma unroll
             for (int r = 0; r < RPL; ++r) v[t][r] = (long long)((unsigned long long)v[t][r] << d);
             cur[t] = s2;
-            if (up == (t == 1)) qrem = q;
+            if (sel == t) qrem = q;
           }
         }
         if (on) {
@@ -545,18 +555,25 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
 #pragma unroll
         for (int t = 0; t < CPL; ++t) g[t] += m[t] >> 29;  // x C / 2^58
         // sum over the LR lanes of a column; with two columns per lane the first exchange
-        // leaves the upper half of the lanes with the second one
+        // leaves the upper half of the lanes with the second one, with three the first two
+        // exchanges leave a quarter of them with each
         long long gt = g[0];
         if constexpr (CPL == 2) {
           const long long send = up ? g[0] : g[1];
           gt = (up ? g[1] : g[0]) + __shfl_xor_sync(kFull, send, kH);
         }
+        if constexpr (CPL == 3) {
+          const bool odd = (lr & kQ) != 0;
+          const long long a = (up ? g[2] : g[0]) + __shfl_xor_sync(kFull, up ? g[0] : g[2], kH);
+          const long long b1 = (up ? 0 : g[1]) + __shfl_xor_sync(kFull, up ? g[1] : 0, kH);
+          gt = (odd ? b1 : a) + __shfl_xor_sync(kFull, odd ? a : b1, kQ);
+        }
 #pragma unroll
-        for (int s = CPL == 2 ? kH / 2 : kH; s >= 1; s >>= 1) gt += __shfl_xor_sync(kFull, gt, s);
-        const int c = cb + lc + (up ? LC : 0);
+        for (int s = CPL == 3 ? kQ / 2 : CPL == 2 ? kH / 2 : kH; s >= 1; s >>= 1) gt += __shfl_xor_sync(kFull, gt, s);
+        const int c = cs;
         const bool on = c > j && c < nc;
         const int2 rD = sb[4 * b], y = sb[4 * b + 1], tq = sb[4 * b + 2];
-        const float qsc = __int_as_float((99 - (up ? cur[CPL - 1] : cur[0])) << 23);  // 2^(-28 - cur)
+        const float qsc = __int_as_float((99 - pick(cur)) << 23);  // 2^(-28 - cur)
         const long long p0 = on ? Rs[ro(j) + c] : 0;
         int h, l;
         fx_limbs((gt + 1) >> 1, h, l);
@@ -570,7 +587,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
         l = (int)((unsigned)nq - ((unsigned)h << 29));
         if (!on) h = l = 0;  // columns up to j are reflectors now
         __syncwarp();        // every lane of a column has read p0
-        if (on && (CPL == 2 ? lr % kH : lr) == 0) Rs[ro(j) + c] = pk;
+        if (on && (CPL == 3 ? lr % kQ : CPL == 2 ? lr % kH : lr) == 0) Rs[ro(j) + c] = pk;
         int qh[CPL], ql[CPL];
         qh[0] = h;
         ql[0] = l;
@@ -580,6 +597,13 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
           ql[0] = up ? ol : l;
           qh[1] = up ? h : oh;
           ql[1] = up ? l : ol;
+        }
+        if constexpr (CPL == 3) {
+#pragma unroll
+          for (int t = 0; t < CPL; ++t) {
+            qh[t] = __shfl_sync(kFull, h, lane - lr + t * kQ);
+            ql[t] = __shfl_sync(kFull, l, lane - lr + t * kQ);
+          }
         }
 #pragma unroll
         for (int r = 0; r < RPL; r += 2) {
@@ -599,7 +623,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
       __syncthreads();
     }
 
-    if constexpr (!KEEP) continue;
+    if (!KEEP) continue;
     // the reflectors' scalars: v = [1; scale x], H = I - tau v v^T, as the apply kernels read
     // them; identities for the rows a piece of a triangle does not reach
     for (int j = tid; j < n; j += 32 * NW) {

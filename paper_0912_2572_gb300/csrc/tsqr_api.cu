@@ -613,6 +613,13 @@ static tsqr_status apply_launch(const tsqr_factors *F, double *B, int64_t ldb, i
   // a tree level whose nodes, four CTAs each, still fit one wave of two CTAs per SM runs
   // 16 columns per CTA: each node's reflector steps get shorter
   const bool narrow = li > 0 && (int64_t)ld.job_count * 4 <= (int64_t)sms * 2;
+  // the tile kernel's time grows with n k, the tensor-core kernel's with panels of 8
+  // reflectors and groups of 8 columns: they cross at n = 12 with 16 columns 0.90 : 1 (24
+  // columns 1.18), n = 16 with 9 0.88 (16: 1.18), n = 24 with 9 0.95 (16: 1.27)
+  if (kg > 8 && kg <= 16 && !formq && pl.n * kg <= 216) {
+    CUDA_TRY(launch_apply_tile(p, ld.job_count, s));
+    return TSQR_OK;
+  }
   if (kg > 8) {
     CUDA_TRY(launch_apply_mma(p, ld.job_count, li == 0 ? pl.tile_h : pl.n, narrow ? 16 : 64, s));
     return TSQR_OK;
@@ -776,6 +783,9 @@ tsqr_status batch_build_on(DeviceInfo di, const tsqr_batch_item *items, int32_t 
     // doubles, whatever the job's own tiles
     int tc = th, cps64 = 0;
     if (!mixed && !factor_tile_choice(it.n, nc, 1 << 20, di.smem_sm, di.reserved, di.optin, 2, tc, cps64)) tc = th;
+    // above 128 columns a tile is a quarter as high: chains of half as many rows (two served
+    // requests of up to 300,000 rows 21.7 ms with the long ones)
+    if (!mixed && nc > 128) tc = 2 * th;
     const int64_t tiles = (it.m + tc - 1) / tc;
     // mixed items: FP32 chains kMixedChainFactor times longer (fewer FP64 tree combines)
     const int64_t Lq = mixed ? (int64_t)L * kMixedChainFactor : L;
@@ -1920,9 +1930,11 @@ tsqr_status tsqr_lstsq(const double *A, int64_t m, int32_t n, int64_t lda, const
   double *W = nullptr;  // Q^T B workspace (m-by-k)
   int32_t *status = nullptr;
   // B's columns are factored along unless they take A's over the edge of the eight-warp job
-  // (64 columns, two CTAs per SM; 1M x 64 with 4 right-hand sides 13.3 ms fused in sixteen
-  // warps): then Q^T B is a pass of its own
-  const bool fused = (n + k) <= 64 || (n > 64 && n + k <= 128);
+  // (64 columns, two CTAs per SM) and there are enough rows for a separate pass of Q^T B to cost
+  // less than the sixteen-warp job does: x 64 with 1 / 4 / 8 right-hand sides, 1,000 rows 1.46 /
+  // 2.01 / 2.68 ms against 1.31 fused, 30,000 2.10 / 2.69 / 3.44 against 2.14, 300,000 4.89 /
+  // 5.88 / 7.09 against 6.75, 1M 9.8 / 11.9 / 14.9 against 15.1
+  const bool fused = (n + k) <= 64 || (n + k <= 128 && (n > 64 || m <= (int64_t)24000 * k));
   st = get_plan(m, n, fused ? n + k : n, leaf_h, arity, flags, f->dp);
   if (st == TSQR_OK) st = factors_alloc(f, s);
   if (st == TSQR_OK) {

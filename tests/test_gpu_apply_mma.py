@@ -86,3 +86,14 @@ def test_non_finite_columns_stay_alone(cuda_lib, bad):
     F.free()
     assert np.all(np.isfinite(Q1[:, :11])) and np.linalg.norm(Q1[:, :11] - Q0[:, :11]) <= 1e-12
     assert not np.any(np.isfinite(Q1[:, 11]))
+
+
+# 9 to 16 columns against few reflectors (n k <= 216: a CTA per job in FP64) and the first
+# widths above it; tiles at the edges of its three heights (128, 256, 512 rows), ragged tails,
+# a last group of 9 columns after 64
+@pytest.mark.parametrize("m,n,k,h,arity,two", [
+    (9, 1, 9, 9, 2, False), (129, 8, 16, 128, 0, True), (513, 13, 16, 256, 0, True), (2049, 24, 9, 512, 0, True),
+    (1537, 12, 15, 512, 4, False), (700, 8, 73, 100, 16, False), (600, 14, 16, 257, 0, True),
+])
+def test_few_reflectors(cuda_lib, m, n, k, h, arity, two):
+    test_matches_the_warp_kernel(cuda_lib, m, n, k, h, arity, two)

@@ -137,3 +137,16 @@ def test_non_finite_entry_in_a_wide_cluster_tree(cuda_lib):
     assert _rel(R[True][:, :c], oracle.r_factor(A)[:, :c]) <= 1e-12
     # row i of R takes column c only at reflector i; reflector c spoils every row from c on
     assert not np.any(np.isfinite(R[True][c, c:])) and not np.any(np.isfinite(R[True][:c, c]))
+
+
+# right-hand sides factored along, or a pass of their own (64 < n + k, m above 24,000 k); chains
+# and tree nodes of 9 to 16 columns on the FP64 job and beside it. Well-conditioned: both
+# solutions are within 1e-12 of the normal one.
+@pytest.mark.parametrize("m,n,k", [(24000, 64, 1), (24001, 64, 1), (48001, 60, 8), (300, 64, 64), (1000, 4, 8),
+                                   (1025, 8, 1), (5000, 8, 8), (3000, 9, 3), (3000, 12, 1), (700, 2, 2)])
+def test_lstsq_routes(cuda_lib, m, n, k):
+    import paper_0912_2572_gb300 as ts
+    A, B = inputs.gaussian(m, n, m + n), inputs.gaussian(m, k, m + k)
+    X = to_host(ts.lstsq(to_dev(A), to_dev(B)))
+    ref = np.linalg.lstsq(A, B, rcond=None)[0]
+    assert np.linalg.norm(X - ref) <= 1e-12 * np.linalg.norm(ref) + 1e-12 * np.linalg.norm(B) / np.linalg.norm(A)
