@@ -1091,7 +1091,7 @@ def bench_ours(args):
                        # times include the time they wait for SMs (alone: config2.apply_qt_k1_ms)
                        "apply_qt_ms_beside_form_q": phase_ms.get("apply_qt", 0) / args.steps,
                        "small_ms": phase_ms.get("small", 0) / args.steps},
-            "roofline": {"kernel": "k_factor (leaf/flat-chain launch)", "bound": "alu", "achieved": achieved,
+            "roofline": {"kernel": "k_factor_fx (leaf/flat-chain launch, 64-bit fixed point)", "bound": "alu", "achieved": achieved,
                          "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                          "traffic": (CHAIN_DRAM_BYTES_PER_ROW_N64 * m if n == 64 else None),
                          "hbm_gbs": (CHAIN_DRAM_BYTES_PER_ROW_N64 * m / (chain_ms * 1e-3) / 1e9 if n == 64 else None),
