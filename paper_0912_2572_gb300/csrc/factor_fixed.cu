@@ -6,8 +6,8 @@
 namespace tsqr {
 namespace {
 
-// A job, or what is left of it once a tile holds an entry the fixed-point form cannot take,
-// which goes through the FP64 job (written for eight warps).
+// A job, or what is left of it once a tile holds an entry the fixed-point form cannot take or
+// is light beside its columns, which goes through the FP64 job (written for eight warps).
 template <int CPL, int LC, int RPL, int NW>
 __device__ __forceinline__ void run_any(const FactorParamsT<double> &p, JobDesc job, unsigned char *smraw) {
   const int done = run_job_fx<CPL, LC, RPL, NW>(p, job, smraw);

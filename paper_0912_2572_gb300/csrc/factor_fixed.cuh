@@ -112,7 +112,25 @@ __device__ __forceinline__ FxRefl fx_reflector(long long alpha, unsigned __int12
   return f;
 }
 
-// Steps between two rescalings of a column.
+// Light tiles. An entry of 2^-s of its column's norm keeps 60 - s bits here, where FP64 keeps
+// 53 of every entry, and what it lost matters once the heavy rows of the column are eliminated:
+// in weighted least squares with the heavy rows first (weights of 1e8 are ordinary for soft
+// constraints) the light rows alone determine the rest of the unknowns. A tile is light in a
+// column, and its job goes on in FP64 from there, if the root mean square of the tile's nonzero
+// entries is below 2^-12 of 2^E, or more of them than a smooth distribution would have (its
+// density at zero is below 1 / rms: eight times that) are below 2^-16. The rows of a chain of
+// M alike rows are at 2^-(1 + log2(M) / 2), so plain chains of up to 2^22 rows stay. A node's
+// triangle falls off along its rows by itself when A is ill-conditioned: there a quarter of the
+// entries may be that small, and the later pieces of a triangle are not looked at. Costs two
+// instructions per entry and tile, beside 37 cycles per entry and step.
+constexpr int kFxLightBits = 16;
+// nz entries, nl of them light, their squares' sum sq 4^d in units of the column's 4^E
+__device__ __forceinline__ bool fx_light(unsigned nz, unsigned nl, float sq, int d, bool tri) {
+  if (nz == 0) return false;
+  const float fz = (float)nz, q = sq * exp2f((float)max(2 * d, -100)) / fz;
+  return q < 0x1p-24f || (float)nl > 4.f + fz * fmaxf(0x1p-13f * rsqrtf(q), tri ? 0.25f : 0.f);
+}
+
 // Shared memory of the job: tails of two reflectors, the next pivot column, scalars (two
 // steps' limbs; every reflector's for the tile's end), column exponents and norms, R and the
 // scales of its row blocks.
@@ -129,8 +147,8 @@ __host__ __device__ constexpr size_t fx_smem_bytes(int n, int nc, int lc, int rp
 // One job. Geometry: CPL columns per lane, LC lane columns, RPL (even) rows per lane; the
 // warp's group has GC = CPL LC columns, a tile at most LR RPL rows with LR = 32 / LC, and
 // nc <= NW GC. Returns the number of tiles done: all of them, or fewer when a tile holds an
-// entry the fixed-point form cannot take (not finite, or outside 2^+-900); the chain's state
-// is then in global memory, where the FP64 job goes on from.
+// entry the fixed-point form cannot take (not finite, or outside 2^+-900) or is light (above);
+// the chain's state is then in global memory, where the FP64 job goes on from.
 //
 // KEEP = false (the batched kernels, which apply nothing later): only R and the right-hand
 // sides' pivot rows are written. A leaf tile is then a triangle-on-tile step from R = 0, so a
@@ -239,6 +257,8 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
       int E = (tt == 0 || c >= nc) ? kFxNone : Es[c];
       float nb = (tt == 0 || c >= nc) ? 0.f : nbs[c];
       rbad[t] = n;
+      float sl = 0.f;  // of the last set: the sum of squares in 4^tl
+      int tl = 0;
       // one set of entries: their largest exponent field, then their squares relative to it
       auto grow = [&](unsigned mx, auto squares) {
 #pragma unroll
@@ -249,7 +269,9 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
         float s = ok ? squares(e) : 0.f;
 #pragma unroll
         for (int m = LR / 2; m >= 1; m >>= 1) s += __shfl_xor_sync(kFull, s, m);
-        if (ok) fx_grow(E, nb, (int)e - 1022, s);
+        sl = s;
+        tl = (int)e - 1022;
+        if (ok) fx_grow(E, nb, tl, s);
       };
       auto habs = [](long long x) { return (unsigned)(x >> 32) & 0x7fffffffu; };
       if (tt == 0 && !zero && !ge) {  // a tree node starts from the first child's triangle
@@ -294,17 +316,28 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
 #pragma unroll
         for (int m = LR / 2; m >= 1; m >>= 1) rbad[t] = min(rbad[t], __shfl_xor_sync(kFull, rbad[t], m));
       }
+      if (off == 0) {
+        const int lim = (E + 1023 - kFxLightBits) * (1 << 20);
+        unsigned cnt = 0;  // entries, and light ones
+#pragma unroll
+        for (int r = 0; r < RPL; ++r) {
+          const unsigned h = habs(v[t][r]);
+          if (h != 0) cnt += (int)h < lim ? 0x10001u : 1u;
+        }
+#pragma unroll
+        for (int m = LR / 2; m >= 1; m >>= 1) cnt += __shfl_xor_sync(kFull, cnt, m);
+        if (E > kFxNone && fx_light(cnt & 0xffff, cnt >> 16, sl, tl - E, tri)) bad = true;
+      }
       En[t] = E;
       nbn[t] = nb;
     }
-    if constexpr (KEEP) {
-      if (__syncthreads_or(bad)) {
-        if (tt > 0) write_r();
-        __threadfence();
-        __syncthreads();
-        return tt;
-      }
-    } else {
+    if (__syncthreads_or(KEEP && bad)) {
+      if (tt > 0) write_r();
+      __threadfence();
+      __syncthreads();
+      return tt;
+    }
+    if constexpr (!KEEP) {
 #pragma unroll
       for (int t = 0; t < CPL; ++t) {
         const int c = cb + lc + LC * t;

@@ -1,0 +1,83 @@
+"""Matrices whose rows differ in scale, the heavy rows first: the order in which Householder
+QR in FP64 keeps the bits of every row (weighted least squares, soft equality constraints).
+Solutions are compared with the exact ones (rational normal equations). A route's error may
+be ten times that of Householder QR in FP64 (the oracle) or of sqrt(n) roundings, whichever
+is larger; work rounded to a fixed fraction of the column's norm is off by the weight times
+2^-61, 1e-11 at a weight of 1e8."""
+import decimal
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_0912_2572_gb300 import inputs
+from conftest import to_dev, to_host
+
+pytestmark = pytest.mark.gpu
+
+
+def _exact(A, B):
+    """argmin ||B - A X|| in 150 digits from the exact normal equations."""
+    def whole(M):
+        out = np.empty(M.shape, dtype=object)
+        out.flat = [int(Fraction(float(x)) * 2 ** 160) for x in M.flat]
+        return out
+
+    a, b = whole(A), whole(B)
+    n, k = A.shape[1], B.shape[1]
+    with decimal.localcontext() as ctx:
+        ctx.prec = 150
+        N = np.concatenate([a.T.dot(a), a.T.dot(b)], axis=1)
+        M = np.empty(N.shape, dtype=object)
+        M.flat = [decimal.Decimal(x) for x in N.flat]
+        for j in range(n):  # Gaussian elimination of a positive definite matrix
+            for i in range(j + 1, n):
+                M[i, j:] -= M[j, j:] * (M[i, j] / M[j, j])
+        X = np.empty((n, k), dtype=object)
+        for i in range(n - 1, -1, -1):
+            for c in range(k):
+                X[i, c] = (M[i, n + c] - sum((M[i, l] * X[l, c] for l in range(i + 1, n)), decimal.Decimal(0))) / M[i, i]
+        return X.astype(np.float64)
+
+
+def _problem(m, n, k, kind, w, seed):
+    """A, B with rows weighted by w: `dense` three heavy rows first; `few` twenty that involve
+    three unknowns only; `falling` all rows, from w down to 1. (A heavy row that is not among
+    the first of its leaf mixes into a light pivot row in FP64 too.)"""
+    A = inputs.gaussian(m, n, seed)
+    B = A @ inputs.gaussian(n, k, seed + 1) + 1e-3 * inputs.gaussian(m, k, seed + 2)
+    s = np.ones(m)
+    if kind == "dense":
+        s[:3] = w
+    elif kind == "falling":
+        s = w ** np.linspace(1, 0, m)
+    else:
+        A[:20, 3:] = 0.0
+        s[:20] = w
+        B[:20] = A[:20] @ inputs.gaussian(n, k, seed + 1)
+    return A * s[:, None], B * s[:, None]
+
+
+def _tolerance(A, B, X):
+    err = np.linalg.norm(oracle.lstsq(A, B) - X) / np.linalg.norm(X)
+    return 10.0 * max(err, 2.0 ** -52 * np.sqrt(A.shape[1]))
+
+
+CASES = [("dense", 1e4), ("dense", 1e8), ("dense", 1e12), ("dense", 1e15), ("few", 1e8), ("few", 1e12),
+         ("falling", 1e10)]
+
+
+@pytest.mark.parametrize("kind,w", CASES)
+@pytest.mark.parametrize("m,n,k", [(900, 6, 2), (900, 24, 1), (1300, 40, 24), (700, 60, 2), (700, 100, 2)])
+def test_weighted_lstsq(cuda_lib, kind, w, m, n, k):
+    """One problem: a flat chain, the two-level tree and the binary tree, right-hand sides
+    factored along."""
+    import paper_0912_2572_gb300 as ts
+    A, B = _problem(m, n, k, kind, w, 10 * n + k)
+    X = _exact(A, B)
+    tol = _tolerance(A, B, X)
+    for kw in ({"arity": 0}, {}, {"leaf_h": max(n, 64), "two_level": False}):
+        Z = to_host(ts.lstsq(to_dev(A), to_dev(B), **kw))
+        err = np.linalg.norm(Z - X) / np.linalg.norm(X)
+        assert err <= tol, (kw, err, tol)
