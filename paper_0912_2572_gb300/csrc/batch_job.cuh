@@ -59,11 +59,11 @@ __device__ __forceinline__ void batch_loop(const BatchParams &bp, unsigned char 
         FactorParamsT<float> fp{};
         fp.A = in.A;
         fp.lda = in.lda;
-        fp.V = static_cast<float *>(in.V);
+        fp.V = in.V;
         fp.ldv = in.ldv;
         fp.tiles = bp.tiles;
-        fp.tau = static_cast<float *>(in.tau);
-        fp.scl = static_cast<float *>(in.scl);
+        fp.tau = in.tau;
+        fp.scl = in.scl;
         fp.n = in.n;
         fp.nc = in.n;
         fp.ldt = in.ldt;
@@ -78,7 +78,7 @@ __device__ __forceinline__ void batch_loop(const BatchParams &bp, unsigned char 
           }
         }
         // hand the chain's triangle to the FP64 tree storage
-        const float *Vs = static_cast<const float *>(in.V) + bj.piv_row;
+        const float *Vs = in.V + bj.piv_row;
         for (int e = threadIdx.x; e < in.n * in.n; e += blockDim.x) {
           const int i = e % in.n, j = e / in.n;
           if (i <= j) in.V64[bj.row64 + i + (int64_t)j * in.ldv64] = (double)__ldcg(Vs + i + (int64_t)j * in.ldv);
@@ -88,10 +88,12 @@ __device__ __forceinline__ void batch_loop(const BatchParams &bp, unsigned char 
         FactorParamsT<double> fp{};
         fp.A = in.A;
         fp.lda = in.lda;
-        fp.V = chain ? static_cast<double *>(in.V) : in.V64;
-        fp.ldv = chain ? in.ldv : in.ldv64;
-        fp.B = in.B;
-        fp.ldb = in.ldb;
+        fp.V = in.V64;
+        fp.ldv = in.ldv64;
+        fp.B = in.B64;
+        fp.ldb = in.ldv64;
+        fp.Bin = in.B;
+        fp.ldbin = in.ldb;
         fp.tiles = bp.tiles;
         fp.n = in.n;
         fp.nc = in.n + in.k;

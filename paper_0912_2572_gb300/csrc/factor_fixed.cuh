@@ -151,7 +151,7 @@ __host__ __device__ constexpr size_t fx_smem_bytes(int n, int nc, int lc, int rp
 // the chain's state is then in global memory, where the FP64 job goes on from.
 //
 // KEEP = false (the batched kernels, which apply nothing later): only R and the right-hand
-// sides' pivot rows are written. A leaf tile is then a triangle-on-tile step from R = 0, so a
+// sides' pivot rows are written, to storage of their own (V and B; the tiles come from A and Bin). A leaf tile is then a triangle-on-tile step from R = 0, so a
 // tile may be shorter than n, and all tiles are done: an entry that is not finite makes the R
 // it would have reached NaN.
 template <int CPL, int LC, int RPL, int NW, bool KEEP = true, bool COH = false>
@@ -227,8 +227,8 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
 #pragma unroll
     for (int t = 0; t < CPL; ++t) {
       const int c = cb + lc + LC * t;
-      const bool in = c < n && !tri;  // from the input A (first touch)
-      const double *src = in ? p.A + r0 + (int64_t)c * p.lda : gptr(r0, c);
+      const bool in = (c < n || !KEEP) && !tri;  // from the inputs (first touch)
+      const double *src = !in ? gptr(r0, c) : c < n ? p.A + r0 + (int64_t)c * p.lda : p.Bin + r0 + (int64_t)(c - n) * p.ldbin;
       const int lim = c >= nc ? 0 : (tri && c < n ? min(ht, c + 1 - off) : ht);
       const bool al = (reinterpret_cast<uintptr_t>(src) & 15) == 0;  // row pairs are 16-byte aligned then
 #pragma unroll

@@ -641,10 +641,10 @@ __device__ __forceinline__ void finish_instance(const BatchInst &in, int64_t row
   }
   if (k > 0 && in.X) {
     double *xs = reinterpret_cast<double *>(smraw);  // n * k
-    const double *C = in.B + row64;                   // (Q^T B)[0:n] in the pivot rows
+    const double *C = in.B64 + row64;                 // (Q^T B)[0:n] in the pivot rows
     for (int e = threadIdx.x; e < n * k; e += blockDim.x) {
       const int i = e % n, c = e / n;
-      xs[e] = __ldcg(C + i + (int64_t)c * in.ldb);
+      xs[e] = __ldcg(C + i + (int64_t)c * in.ldv64);
     }
     __syncthreads();
     for (int i = n - 1; i >= 0; --i) {

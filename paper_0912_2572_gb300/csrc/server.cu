@@ -558,7 +558,7 @@ tsqr_status tsqr_server_submit(tsqr_server *S, const tsqr_batch_item *item, int6
   if (!S || !item) return TSQR_ERR_ARG;
   tsqr_status st = tsqr::check_batch_item(*item, 0);
   if (st != TSQR_OK) return st;
-  SrvReq r{*item, 0, Clock::now(), tsqr::batch_item_bytes(*item), nullptr};
+  SrvReq r{*item, 0, Clock::now(), tsqr::batch_item_bytes(*item, S->chain_tiles), nullptr};
   if (S->res) {  // plan now: a request the resident kernel cannot run is refused here
     PlanPtr p(new (std::nothrow) tsqr::ResidentPlan(), PlanFree());
     if (!p) return TSQR_ERR_OOM;

@@ -389,8 +389,9 @@ static tsqr_status make_plan_on(const DeviceInfo &di, Plan &pl, int64_t m, int n
     const int64_t cl_cps = std::min<int64_t>(nc > 64 ? 2 : 3, (int64_t)(di.smem_sm / (csm + di.reserved + 1024)));
     if ((pl.flags & TSQR_CLUSTER) && pl.arity == 2 && !mixed && csm > 0 && cl_cps >= 1)
       plan_clusters(pl, (int64_t)di.sms * cl_cps);
-    if (mixed) {
-      // the tree works on a compact FP64 array: chain c's pivot block at rows c*n..c*n+n-1
+    if (max_cps == 2) {
+      // batched: the tree works on a compact FP64 array, chain c's pivot block at rows
+      // c*n..c*n+n-1
       std::vector<std::pair<int64_t, int64_t>> idx;  // (global pivot row, chain)
       const int32_t G = pl.launches[0].job_count;
       for (int32_t c = 0; c < G; ++c) idx.push_back({pl.jobs[c].piv_row, c});
@@ -724,7 +725,7 @@ struct BatchBuild {
   std::vector<TileDesc> tiles;
   std::vector<int64_t> root;  // where each item's R lands in its tree storage
   struct Off {
-    size_t V, B, tau, scl, V64, tau64, scl64;
+    size_t V, tau, scl, V64, B64;
   };
   std::vector<Off> offs;
   size_t o_inst = 0, o_jobs = 0, o_tiles = 0, o_cnt = 0, o_st = 0;
@@ -855,7 +856,7 @@ tsqr_status batch_build_on(DeviceInfo di, const tsqr_batch_item *items, int32_t 
     std::vector<std::pair<int64_t, int32_t>> rowkey(G);  // (tree-storage row, chain index)
     for (int32_t c = 0; c < G; ++c) {
       holder[c] = c;
-      rowkey[c] = {pl.mixed ? (int64_t)c * pl.n : pl.jobs[c].piv_row, c};
+      rowkey[c] = {(int64_t)c * pl.n, c};
     }
     std::sort(rowkey.begin(), rowkey.end());
     auto chain_of = [&](int64_t row) {
@@ -864,8 +865,8 @@ tsqr_status batch_build_on(DeviceInfo di, const tsqr_batch_item *items, int32_t 
     for (int32_t c = 0; c < G; ++c) {
       BatchJob &bj = b.jobs[gidx[q][c]];
       const JobDesc &jd = pl.jobs[c];
-      bj.piv_row = jd.piv_row;
-      bj.row64 = pl.mixed ? (int64_t)c * pl.n : jd.piv_row;
+      bj.row64 = (int64_t)c * pl.n;
+      bj.piv_row = pl.mixed ? jd.piv_row : bj.row64;
       bj.tile_begin = (int32_t)(tile_base[q] + jd.tile_begin);
       bj.tile_count = jd.tile_count;
       bj.inst = q;
@@ -908,19 +909,17 @@ tsqr_status batch_build_on(DeviceInfo di, const tsqr_batch_item *items, int32_t 
   for (int32_t q = 0; q < count; ++q) {
     const tsqr_batch_item &it = items[q];
     const Plan &pl = b.plans[q];
-    const size_t elem = pl.mixed ? sizeof(float) : sizeof(double);
-    const size_t nrefl = pl.tiles.size() * (size_t)it.n;
+    const size_t Gn = (size_t)pl.launches[0].job_count * it.n;
     BatchBuild::Off &o = b.offs[q];
     o = {};
-    o.V = take(elem * (size_t)it.m * it.n);
-    o.B = (!pl.mixed && it.k > 0) ? take(sizeof(double) * (size_t)it.m * it.k) : 0;
-    o.tau = take(elem * nrefl);
-    o.scl = take(elem * nrefl);
-    if (pl.mixed) {
-      const int64_t Gn = (int64_t)pl.launches[0].job_count * it.n;
-      o.V64 = take(sizeof(double) * (size_t)Gn * it.n);
-      o.tau64 = take(sizeof(double) * nrefl);
-      o.scl64 = take(sizeof(double) * nrefl);
+    o.V64 = take(sizeof(double) * Gn * it.n);
+    if (pl.mixed) {  // the FP32 chains keep their reflectors
+      const size_t nrefl = pl.tiles.size() * (size_t)it.n;
+      o.V = take(sizeof(float) * (size_t)it.m * it.n);
+      o.tau = take(sizeof(float) * nrefl);
+      o.scl = take(sizeof(float) * nrefl);
+    } else if (it.k > 0) {
+      o.B64 = take(sizeof(double) * Gn * it.k);
     }
   }
   b.o_inst = take(sizeof(BatchInst) * count);
@@ -984,21 +983,13 @@ void batch_bind(BatchBuild &b, char *base) {
     bi = {};
     bi.A = it.A;
     bi.lda = it.lda;
-    bi.V = base + o.V;
-    bi.ldv = it.m;
-    bi.ldb = it.m;
-    bi.tau = base + o.tau;
-    bi.scl = base + o.scl;
+    bi.V64 = (double *)(base + o.V64);
+    bi.ldv64 = (int64_t)pl.launches[0].job_count * it.n;
     if (pl.mixed) {
-      bi.V64 = (double *)(base + o.V64);
-      bi.ldv64 = (int64_t)pl.launches[0].job_count * it.n;
-      bi.tau64 = (double *)(base + o.tau64);
-      bi.scl64 = (double *)(base + o.scl64);
-    } else {
-      bi.V64 = (double *)bi.V;
-      bi.ldv64 = it.m;
-      bi.tau64 = (double *)bi.tau;
-      bi.scl64 = (double *)bi.scl;
+      bi.V = (float *)(base + o.V);
+      bi.ldv = it.m;
+      bi.tau = (float *)(base + o.tau);
+      bi.scl = (float *)(base + o.scl);
     }
     bi.R = it.R;
     bi.ldr = it.ldr;
@@ -1007,7 +998,11 @@ void batch_bind(BatchBuild &b, char *base) {
     bi.status = (int32_t *)(base + b.o_st) + q;
     bi.n = it.n;
     bi.k = pl.mixed ? 0 : it.k;
-    bi.B = bi.k > 0 ? (double *)(base + o.B) : nullptr;
+    if (bi.k > 0) {
+      bi.B = it.B;
+      bi.ldb = it.ldb;
+      bi.B64 = (double *)(base + o.B64);
+    }
     bi.ldt = pl.tile_h;
     bi.mixed = pl.mixed ? 1 : 0;
     bi.wy = b.wy[q];
@@ -1041,17 +1036,10 @@ tsqr_status batch_upload(const BatchBuild &b, char *base, cudaStream_t s) {
   return TSQR_OK;
 }
 
-// One run: the right-hand-side copies, counter and flag resets, the persistent kernel,
+// One run: counter and flag resets, the persistent kernel,
 // and the refinement launches. Device-side operations only, so it can be captured in a
 // CUDA graph.
 tsqr_status batch_enqueue(const BatchBuild &b, char *base, cudaStream_t s, bool profile) {
-  for (int32_t q = 0; q < b.count; ++q) {
-    const tsqr_batch_item &it = b.items[q];
-    const BatchInst &bi = b.inst[q];
-    if (bi.k > 0)
-      CUDA_TRY(cudaMemcpy2DAsync(bi.B, sizeof(double) * it.m, it.B, sizeof(double) * it.ldb, sizeof(double) * it.m,
-                                 it.k, cudaMemcpyDeviceToDevice, s));
-  }
   CUDA_TRY(cudaMemsetAsync(base + b.o_cnt, 0, sizeof(int32_t) * ((size_t)b.njobs + 1), s));
   CUDA_TRY(cudaMemsetAsync(base + b.o_st, 0, sizeof(int32_t) * b.count, s));
   if (!b.rinst.empty()) {
@@ -1248,9 +1236,6 @@ tsqr_status tsqr::resident_upload(const ResidentPlan &p, char *base, cudaStream_
   if (st != TSQR_OK) return st;
   const tsqr_batch_item &it = b.items[0];
   const BatchInst &bi = b.inst[0];
-  if (bi.k > 0)
-    CUDA_TRY(cudaMemcpy2DAsync(bi.B, sizeof(double) * it.m, it.B, sizeof(double) * it.ldb, sizeof(double) * it.m,
-                               it.k, cudaMemcpyDeviceToDevice, s));
   // counters, status and flags are cleared by copies (copy engines), never by kernels: the
   // resident kernel may hold every SM while these run
   int32_t *pending = (int32_t *)(base + b.bytes);
@@ -1360,12 +1345,16 @@ int32_t tsqr::resolve_batch_prec(const tsqr_batch_item &it) {
   return mixed < fp64 ? TSQR_MIXED : TSQR_FP64;
 }
 
-size_t tsqr::batch_item_bytes(const tsqr_batch_item &it) {
+size_t tsqr::batch_item_bytes(const tsqr_batch_item &it, int32_t chain_tiles) {
   const bool mixed = resolve_batch_prec(it) == TSQR_MIXED;
   const size_t m = (size_t)it.m, n = (size_t)it.n, k = (size_t)it.k;
   if (mixed)  // FP32 chains, FP64 tree blocks, refinement partials
     return 4 * m * n + 8 * (m / 64 + 1) * n + 8 * (m / kRefineRows + 1) * n * k + n * n * 64 + 65536;
-  return 8 * m * n + 8 * m * k + n * n * 64 + 65536;
+  // the chains' triangles and right-hand-side rows, and the tables (a chain has at most one
+  // tile more than chain_tiles tiles, rounded, of at least batch_job_rows rows)
+  const size_t L = chain_tiles > 0 ? (size_t)chain_tiles : 8, tiles = m / (size_t)batch_job_rows((int)(n + k)) + 1;
+  const size_t G = (tiles + L / 2) / L + 1;
+  return 8 * G * n * (n + k) + 64 * (tiles + 4 * G) + n * n * 64 + 65536;
 }
 
 const char *tsqr::last_error_text() { return g_last_error.c_str(); }

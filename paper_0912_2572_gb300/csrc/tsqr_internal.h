@@ -132,6 +132,8 @@ struct FactorParamsT {
   int64_t ldv;
   R *B;             // optional extra columns (Q^T B fused), m-by-(nc-n), in place
   int64_t ldb;
+  const double *Bin;  // batched FP64 chains: the right-hand sides' first-touch input (B then
+  int64_t ldbin;      // holds the pivot rows only, like V)
   const JobDesc *jobs;
   const TileDesc *tiles;
   R *tau;
@@ -179,14 +181,14 @@ bool factor_tile_choice(int n, int nc, int leaf_h, size_t smem_per_sm, size_t re
 struct BatchInst {
   const double *A;  // input, m-by-n, leading dimension lda
   int64_t lda;
-  void *V;          // chain storage: double (FP64) or float (mixed), m-by-n, ld = ldv
-  int64_t ldv;
-  double *B;        // fused right-hand sides (library copy, m-by-k) or null
+  const double *B;  // fused right-hand sides (input, m-by-k) or null
   int64_t ldb;
-  void *tau, *scl;  // chain reflector scalars (same element type as V)
-  double *V64;      // tree storage: V itself (FP64) or the compact pivot blocks (mixed)
+  float *V;         // mixed items: FP32 chain storage, m-by-n, ld = ldv
+  int64_t ldv;
+  float *tau, *scl; // and its reflector scalars
+  double *V64;      // tree storage, chain c's triangle at rows c n..: n columns
   int64_t ldv64;
-  double *tau64, *scl64;
+  double *B64;      // and the right-hand sides' pivot rows: k columns, the same rows
   double *R;        // optional output, n-by-n
   int64_t ldr;
   double *X;        // optional output, n-by-k
@@ -198,7 +200,7 @@ struct BatchInst {
 };
 
 struct BatchJob {   // chain jobs first (queue order), then tree nodes
-  int64_t piv_row;  // pivot rows in the job's storage (V for chains, V64 for nodes)
+  int64_t piv_row;  // pivot rows in the job's storage (V for FP32 chains, else V64)
   int64_t row64;    // where the job's triangle lives in the tree storage
   int32_t tile_begin, tile_count;
   int32_t inst, parent;  // parent node (job index) or -1 at the root
@@ -378,7 +380,7 @@ tsqr_status batch_solve_internal(const tsqr_batch_item *items, int32_t count, in
                                  cudaStream_t s, int32_t *status, int32_t *status_async, double *info,
                                  int32_t ctas_per_sm = 0);
 tsqr_status check_batch_item(const tsqr_batch_item &it, int32_t q);
-size_t batch_item_bytes(const tsqr_batch_item &it);  // device workspace estimate for admission
+size_t batch_item_bytes(const tsqr_batch_item &it, int32_t chain_tiles);  // device workspace estimate for admission
 int32_t resolve_batch_prec(const tsqr_batch_item &it);  // TSQR_FP64 or TSQR_MIXED
 const char *last_error_text();
 size_t live_free_bytes();  // device memory free now, counting the pool's unused reserve

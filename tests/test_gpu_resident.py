@@ -189,3 +189,21 @@ def test_resident_rings_wrap_around(cuda_lib):
         if i % 8 == 0:
             A, B = reqs[i]
             assert rel(to_host(X), oracle.lstsq(A, B)) <= 1e-10
+
+
+@pytest.mark.parametrize("m,n,k", [(60_000, 64, 2), (40_000, 100, 0), (200_000, 8, 8)])
+def test_fp64_requests_take_their_triangles_only(cuda_lib, m, n, k):
+    """An FP64 request keeps each chain's triangle and the rows of its right-hand sides, not
+    reflectors or copies of its inputs: it fits an arena of half the size of A and B."""
+    import paper_0912_2572_gb300 as ts
+    A, B = inputs.gaussian(m, n, m), inputs.gaussian(m, max(k, 1), m + 1)
+    item = _item(A, B if k else None)
+    with ts.Server(resident=True, max_bytes=4 * m * (n + k), ctas_per_sm=1) as srv:
+        _, (R, X) = srv.submit(item)
+        srv.drain()
+        (_, _, st), = srv.poll()
+    assert st == 0
+    Ra, Xa = _alone(item, 0)
+    assert np.array_equal(to_host(R), Ra)
+    if k:
+        assert np.array_equal(to_host(X), Xa)
