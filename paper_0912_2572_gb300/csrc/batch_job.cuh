@@ -14,30 +14,42 @@ namespace {
 // height (a 512-row tile's registers would all be walked for 16 rows). CHAINS: the launch has
 // FP64 items; without their builds the kernel's other jobs compile better (16.7M x 32 mixed:
 // the factorization 10.4 ms, 11.5 beside them).
+//
+// What a light tile leaves of a job goes through the FP64 job, out of line: it is rare, and
+// inlined it would cost the kernel's other jobs registers.
+template <int CMAX, bool COH>
+__device__ __noinline__ void run_rest_fp64(const FactorParamsT<double> p, JobDesc job, int done, unsigned char *smraw) {
+  job.tile_begin += done;
+  job.tile_count -= done;
+  run_job<CMAX, COH, false>(p, job, smraw);
+}
+
 template <int CMAX, bool CHAINS, bool COH>
 __device__ __forceinline__ void run_batch_job(const FactorParamsT<double> &p, const JobDesc job, unsigned char *smraw,
                                               bool node) {
   constexpr int NW = kThreads / 32;
+  int done = 0;
   if (p.nc <= 16) {
-    if (node) run_job_fx<2, 1, 2, NW, false, COH>(p, job, smraw);
-    else if constexpr (CHAINS) run_job_fx<2, 1, 16, NW, false, COH>(p, job, smraw);
+    if (node) done = run_job_fx<2, 1, 2, NW, false, COH>(p, job, smraw);
+    else if constexpr (CHAINS) done = run_job_fx<2, 1, 16, NW, false, COH>(p, job, smraw);
   } else if (p.nc <= 32) {
     if constexpr (CMAX >= 2) {
-      if (node) run_job_fx<2, 2, 2, NW, false, COH>(p, job, smraw);
-      else if constexpr (CHAINS) run_job_fx<2, 2, 18, NW, false, COH>(p, job, smraw);
+      if (node) done = run_job_fx<2, 2, 2, NW, false, COH>(p, job, smraw);
+      else if constexpr (CHAINS) done = run_job_fx<2, 2, 18, NW, false, COH>(p, job, smraw);
     }
   } else if (p.nc <= 64) {
     if constexpr (CMAX >= 4) {
-      if (node) run_job_fx<2, 4, 8, NW, false, COH>(p, job, smraw);
-      else if constexpr (CHAINS) run_job_fx<2, 4, 18, NW, false, COH>(p, job, smraw);
+      if (node) done = run_job_fx<2, 4, 8, NW, false, COH>(p, job, smraw);
+      else if constexpr (CHAINS) done = run_job_fx<2, 4, 18, NW, false, COH>(p, job, smraw);
     }
   } else if (p.nc <= 96) {
-    if constexpr (CMAX >= 8) run_job_fx<3, 4, 12, NW, false, COH>(p, job, smraw);
+    if constexpr (CMAX >= 8) done = run_job_fx<3, 4, 12, NW, false, COH>(p, job, smraw);
   } else if (p.nc <= 128) {
-    if constexpr (CMAX >= 8) run_job_fx<2, 8, 18, NW, false, COH>(p, job, smraw);
+    if constexpr (CMAX >= 8) done = run_job_fx<2, 8, 18, NW, false, COH>(p, job, smraw);
   } else {
-    if constexpr (CMAX >= 16 && CHAINS) run_job_fx<3, 8, 14, NW, false, COH>(p, job, smraw);
+    if constexpr (CMAX >= 16 && CHAINS) done = run_job_fx<3, 8, 14, NW, false, COH>(p, job, smraw);
   }
+  if (done < job.tile_count) run_rest_fp64<CMAX, COH>(p, job, done, smraw);
 }
 
 // Items of the batched kernels (bp of k_factor_batch), see factor.cu.
@@ -97,6 +109,7 @@ __device__ __forceinline__ void batch_loop(const BatchParams &bp, unsigned char 
         fp.tiles = bp.tiles;
         fp.n = in.n;
         fp.nc = in.n + in.k;
+        fp.ldt = in.ldt64;
         run_batch_job<CMAX, CHAINS, false>(fp, jd, smraw, !chain);
       }
       if (bj.parent < 0) {

@@ -89,12 +89,17 @@ cudaError_t launch_factor_batch(const BatchParams &p, int cmax, int grid, size_t
   return launch_batch_kernel(k_factor_batch<4, true>, p, grid, smem_bytes, s);
 }
 
-size_t batch_job_smem(int n, int nc) {
-  if (nc <= 16) return fx_smem_bytes(n, nc, 1, 16);
-  if (nc <= 32) return fx_smem_bytes(n, nc, 2, 18);
-  if (nc <= 64) return fx_smem_bytes(n, nc, 4, 18);
-  if (nc <= 96) return fx_smem_bytes(n, nc, 4, 12);
-  return nc <= 128 ? fx_smem_bytes(n, nc, 8, 18) : fx_smem_bytes(n, nc, 8, 14);
+size_t batch_job_smem(int n, int nc, bool node) {
+  const size_t fx = nc <= 16   ? fx_smem_bytes(n, nc, 1, 16)
+                    : nc <= 32 ? fx_smem_bytes(n, nc, 2, 18)
+                    : nc <= 64 ? fx_smem_bytes(n, nc, 4, 18)
+                    : nc <= 96 ? fx_smem_bytes(n, nc, 4, 12)
+                               : fx_smem_bytes(n, nc, 8, nc <= 128 ? 18 : 14);
+  return std::max(fx, factor_smem_bytes(nc, batch_job_ldt(n, nc, node)));
+}
+int batch_job_ldt(int n, int nc, bool node) {
+  const int rows = batch_job_rows(nc), pieces = (n + rows - 1) / rows;  // as split_tree_tiles
+  return node ? (n + pieces - 1) / pieces : rows;
 }
 
 int batch_job_rows(int nc) {

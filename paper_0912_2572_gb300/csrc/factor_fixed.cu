@@ -15,7 +15,7 @@ __device__ __forceinline__ void run_any(const FactorParamsT<double> &p, JobDesc 
     job.tile_begin += done;
     job.tile_count -= done;
     if (NW == 8 || threadIdx.x < kThreads)
-      run_job<(NW > 8 ? 8 : LC == 1 ? 1 : LC == 2 ? 2 : 4), true>(p, job, smraw, NW > 8);
+      run_job<(NW > 8 ? 8 : LC == 1 ? 1 : LC == 2 ? 2 : 4)>(p, job, smraw, NW > 8);
   }
 }
 
@@ -78,7 +78,7 @@ cudaError_t launch_fx_cluster(FactorParamsT<double> p, const ClusterSlot *slots,
 // CTAs per SM fit at 64 registers.
 __global__ void __launch_bounds__(kThreads, 4) k_factor_narrow(const FactorParamsT<double> p) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  run_job<1, true>(p, p.jobs[p.job0 + blockIdx.x], smraw);
+  run_job<1>(p, p.jobs[p.job0 + blockIdx.x], smraw);
 }
 
 cudaError_t launch_narrow(const FactorParamsT<double> &p, int njobs, cudaStream_t s) {

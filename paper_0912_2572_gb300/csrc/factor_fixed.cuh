@@ -151,9 +151,10 @@ __host__ __device__ constexpr size_t fx_smem_bytes(int n, int nc, int lc, int rp
 // the chain's state is then in global memory, where the FP64 job goes on from.
 //
 // KEEP = false (the batched kernels, which apply nothing later): only R and the right-hand
-// sides' pivot rows are written, to storage of their own (V and B; the tiles come from A and Bin). A leaf tile is then a triangle-on-tile step from R = 0, so a
-// tile may be shorter than n, and all tiles are done: an entry that is not finite makes the R
-// it would have reached NaN.
+// sides' pivot rows are written, to storage of their own (V and B; the tiles come from A and
+// Bin). A leaf tile is then a triangle-on-tile step from R = 0, so a tile may be shorter than
+// n, and only light tiles end the job early: an entry that is not finite makes the R it would
+// have reached NaN.
 template <int CPL, int LC, int RPL, int NW, bool KEEP = true, bool COH = false>
 __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const JobDesc job, unsigned char *smraw) {
   constexpr int GC = CPL * LC, LR = 32 / LC, kRpw = (LR * RPL + 31) / 32, kRows = 32 * kRpw;
@@ -331,7 +332,7 @@ __device__ __forceinline__ int run_job_fx(const FactorParamsT<double> &p, const 
       En[t] = E;
       nbn[t] = nb;
     }
-    if (__syncthreads_or(KEEP && bad)) {
+    if (__syncthreads_or(bad)) {
       if (tt > 0) write_r();
       __threadfence();
       __syncthreads();

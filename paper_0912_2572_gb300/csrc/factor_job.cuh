@@ -195,17 +195,19 @@ __device__ __forceinline__ void bar_arrive_n(int id, int count) {
   asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
 
-// EARLY_PF: the scalar warp loads the next pivot row at the start of the step (its L2
-// latency overlaps the norm and the reflector, which matters on tree nodes, where the
-// update is short) instead of after the coefficients (fewer live registers: the resident
-// kernel, at its register cap, keeps that order). The row is not written before step j+1,
-// so both orders load the same values and give bitwise the same results.
+// The scalar warp loads the next pivot row at the start of the step (its L2 latency overlaps
+// the norm and the reflector, which matters on tree nodes, where the update is short; the row
+// is not written before step j+1).
 //
 // part: the CTA has more threads than the kThreads that run the job.
 //
+// KEEP = false (the batched kernels, as in factor_fixed.cuh): the right-hand sides come from
+// Bin, only R and the right-hand sides' pivot rows are written, and a leaf tile may have fewer
+// rows than n (the reflectors it has no row for are left to the next tile: R's rows are zero).
+//
 // COH: inputs and descriptors are read through L2 only (the resident kernel, whose inputs
 // and tables change while it runs); otherwise A goes through the read-only cache.
-template <int CMAX, bool EARLY_PF, bool COH = false>
+template <int CMAX, bool COH = false, bool KEEP = true>
 __device__ __forceinline__ void run_job(const FactorParamsT<double> &p, const JobDesc job, unsigned char *smraw,
                                         bool part = false) {
   using R = double;
@@ -247,8 +249,8 @@ __device__ __forceinline__ void run_job(const FactorParamsT<double> &p, const Jo
     // stage the tile: GEQRT/TSQRT tiles come from A (first touch), TTQRT from V
     for (int c = warp; c < nc; c += kThreads / 32) {
       R *dst = T + (size_t)c * ldt;
-      if (c < n && kind != TTQRT) {
-        const double *src = p.A + r0 + (int64_t)c * p.lda;
+      if ((c < n || !KEEP) && kind != TTQRT) {
+        const double *src = c < n ? p.A + r0 + (int64_t)c * p.lda : p.Bin + r0 + (int64_t)(c - n) * p.ldbin;
         warp_copy(dst, src, ht, lane, [](const double *q) { return ld_input<COH>(q); },
                   [](const double2 *q) { return ld_input<COH>(q); });
       } else {
@@ -259,13 +261,14 @@ __device__ __forceinline__ void run_job(const FactorParamsT<double> &p, const Jo
     }
     if (!ge)
       for (int c = tid; c < nc; c += kThreads) PV[c] = (c >= j0) ? __ldcg(piv_ptr(j0, c)) : R(0);
-    for (int j = tid; j < j0; j += kThreads) {  // identity reflectors
+    for (int j = tid; KEEP && j < j0; j += kThreads) {  // identity reflectors
       p.tau[td.refl + j] = R(0);
       p.scl[td.refl + j] = R(0);
     }
     sync();
 
-    for (int j = j0; j < n; ++j) {
+    const int jend = !KEEP && ge ? min(n, ht) : n;
+    for (int j = j0; j < jend; ++j) {
       int lo, hi;
       refl_rows(kind, j, ht, lo, hi, off);
       if (!sw) {
@@ -280,7 +283,7 @@ __device__ __forceinline__ void run_job(const FactorParamsT<double> &p, const Jo
         // overlaps this step's norm and reflector
         R pf[PCN];
         const bool do_pf = !ge && j + 1 < n;
-        if (EARLY_PF && do_pf) {
+        if (do_pf) {
 #pragma unroll
           for (int q = 0; q < PCN; ++q) {
             const int c = j + 1 + lane + 32 * q;
@@ -331,14 +334,16 @@ __device__ __forceinline__ void run_job(const FactorParamsT<double> &p, const Jo
             T[(size_t)j * ldt + j] = rf.beta;
           else
             *piv_ptr(j, j) = rf.beta;
-          p.tau[td.refl + j] = rf.tau;
-          p.scl[td.refl + j] = rf.scale;
+          if (KEEP) {
+            p.tau[td.refl + j] = rf.tau;
+            p.scl[td.refl + j] = rf.scale;
+          }
         }
         if (do_pf) {
 #pragma unroll
           for (int q = 0; q < PCN; ++q) {
             const int c = j + 1 + lane + 32 * q;
-            if (c < nc) PV[c] = EARLY_PF ? pf[q] : __ldcg(piv_ptr(j + 1, c));
+            if (c < nc) PV[c] = pf[q];
           }
         }
         __syncwarp();
@@ -346,10 +351,13 @@ __device__ __forceinline__ void run_job(const FactorParamsT<double> &p, const Jo
       sync();
     }
 
+    if (!KEEP && ge)  // the leaf's R to the pivot rows
+      for (int c = warp; c < nc; c += kThreads / 32)
+        for (int i = lane; i < (c < n ? c + 1 : n); i += 32) *piv_ptr(i, c) = i < ht ? T[(size_t)c * ldt + i] : R(0);
     // write the tile back: GEQRT -> R above / V below the diagonal, TSQRT -> dense
     // reflector tails, TTQRT -> the upper triangle only (the child's own leaf
     // reflectors live below its diagonal)
-    for (int c = warp; c < nc; c += kThreads / 32) {
+    for (int c = warp; KEEP && c < nc; c += kThreads / 32) {
       R *dst = (c < n) ? p.V + r0 + (int64_t)c * p.ldv : p.B + r0 + (int64_t)(c - n) * p.ldb;
       const R *src = T + (size_t)c * ldt;
       const int lim = (kind == TTQRT && c < n) ? max(0, min(ht, c + 1 - off)) : ht;

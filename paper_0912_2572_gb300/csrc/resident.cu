@@ -165,9 +165,19 @@ __device__ void signal_done(const ResParams &p, int slot, const ResItemDev &it) 
   }
 }
 
+__device__ __forceinline__ void run_chain_f32(const FactorParamsT<float> fp, const JobDesc jd, unsigned char *smraw) {
+  switch (fp.n <= 16 ? 1 : (fp.n <= 32 ? 2 : (fp.n <= 64 ? 4 : 8))) {
+    case 1: run_job_f32s<1, true>(fp, jd, smraw); break;
+    case 2: run_job_f32s<2, true>(fp, jd, smraw); break;
+    case 4: run_job_f32s<4, true>(fp, jd, smraw); break;
+    default: run_job_f32s<8, true>(fp, jd, smraw); break;
+  }
+}
+
 // A chain job of the request in `slot`, then every tree node it is the last child of (the
-// batched kernel's climb), then, at the root, R and X or the first refinement step.
-__device__ void run_chain(const ResParams &p, int slot, int jb, unsigned char *smraw, int *s_go,
+// batched kernel's climb), then, at the root, R and X or the first refinement step. Inlined:
+// under the function ABI the jobs' register tiles spilled 2 to 3.8 KB.
+__device__ __forceinline__ void run_chain(const ResParams &p, int slot, int jb, unsigned char *smraw, int *s_go,
                           unsigned long long *s_base) {
   const ResItemDev it = ldcg_struct(p.items + slot);
   const BatchInst &in = it.inst;
@@ -187,12 +197,7 @@ __device__ void run_chain(const ResParams &p, int slot, int jb, unsigned char *s
       fp.n = in.n;
       fp.nc = in.n;
       fp.ldt = in.ldt;
-      switch (in.n <= 16 ? 1 : (in.n <= 32 ? 2 : (in.n <= 64 ? 4 : 8))) {
-        case 1: run_job_f32s<1, true>(fp, jd, smraw); break;
-        case 2: run_job_f32s<2, true>(fp, jd, smraw); break;
-        case 4: run_job_f32s<4, true>(fp, jd, smraw); break;
-        default: run_job_f32s<8, true>(fp, jd, smraw); break;
-      }
+      run_chain_f32(fp, jd, smraw);
       // hand the chain's triangle to the FP64 tree storage
       const float *Vs = in.V + bj.piv_row;
       for (int e = threadIdx.x; e < in.n * in.n; e += blockDim.x) {
@@ -213,6 +218,7 @@ __device__ void run_chain(const ResParams &p, int slot, int jb, unsigned char *s
       fp.tiles = it.tiles;
       fp.n = in.n;
       fp.nc = in.n + in.k;
+      fp.ldt = in.ldt64;
       run_batch_job<kResCmax, true, true>(fp, jd, smraw, !chain);
     }
     if (bj.parent < 0) {

@@ -808,7 +808,7 @@ tsqr_status batch_build_on(DeviceInfo di, const tsqr_batch_item *items, int32_t 
       }
     }
     b.smem = std::max(b.smem, chain_smem);
-    b.smem = std::max(b.smem, batch_job_smem(it.n, nc));
+    b.smem = std::max(b.smem, batch_job_smem(it.n, nc, mixed));
     b.smem = std::max(b.smem, sizeof(double) * (size_t)it.n * std::max(it.k, 1));
     while (16 * b.cmax < nc) b.cmax *= 2;
     cps_min = std::min(cps_min, b.plans[q].ctas_per_sm);
@@ -1004,6 +1004,7 @@ void batch_bind(BatchBuild &b, char *base) {
       bi.B64 = (double *)(base + o.B64);
     }
     bi.ldt = pl.tile_h;
+    bi.ldt64 = batch_job_ldt(it.n, pl.nc, pl.mixed);
     bi.mixed = pl.mixed ? 1 : 0;
     bi.wy = b.wy[q];
   }
@@ -1208,7 +1209,7 @@ tsqr_status tsqr::resident_plan(const tsqr_batch_item &it, int32_t chain_tiles, 
     const int nc = b->plans[q].mixed ? it.n : it.n + it.k;
     const size_t elem = b->plans[q].mixed ? sizeof(float) : sizeof(double);
     if (b->plans[q].mixed) smem = std::max(smem, factor_smem_bytes(nc, b->plans[q].tile_h, elem));
-    smem = std::max(smem, batch_job_smem(it.n, nc));
+    smem = std::max(smem, batch_job_smem(it.n, nc, b->plans[q].mixed));
     // FP64 requests whose n rows of doubles do not fit two CTAs per SM are admitted at one
     // only (they need less since the job keeps its tile in registers; the rule is kept)
     if (!b->plans[q].mixed) smem = std::max(smem, factor_smem_bytes(nc, it.n, sizeof(double)));

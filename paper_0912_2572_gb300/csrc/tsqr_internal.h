@@ -195,6 +195,7 @@ struct BatchInst {
   int64_t ldx;
   int32_t *status;  // device flag set to 4 when R is singular (solve only)
   int32_t n, k, ldt, mixed;
+  int32_t ldt64;     // rows of the tallest tile of its FP64 jobs (chains of FP64 items, nodes)
   int32_t wy;        // mixed items: FP32 chains by compact-WY panels with 3xTF32 tensor-core
                      // updates (run_job_f32wy) instead of the unblocked register tile
 };
@@ -217,8 +218,9 @@ struct BatchParams {
 };
 
 // Shared memory and tallest tile of an FP64 job of the batched kernels (nc columns, n of them
-// the matrix's); a tile may be shorter than n.
-size_t batch_job_smem(int n, int nc);
+// the matrix's); a tile may be shorter than n. node: tree nodes only (mixed items).
+size_t batch_job_smem(int n, int nc, bool node);
+int batch_job_ldt(int n, int nc, bool node);
 int batch_job_rows(int nc);
 cudaError_t launch_factor_batch_wide(const BatchParams &p, int grid, size_t smem_bytes, cudaStream_t s,
                                      bool fp64_items, bool wy);

@@ -81,3 +81,45 @@ def test_weighted_lstsq(cuda_lib, kind, w, m, n, k):
         Z = to_host(ts.lstsq(to_dev(A), to_dev(B), **kw))
         err = np.linalg.norm(Z - X) / np.linalg.norm(X)
         assert err <= tol, (kw, err, tol)
+
+
+# leaves of one and of several tiles (512, 288, 144, 96, 72 and 56 rows by width), tiles
+# shorter than n, one chain and several with tree nodes
+@pytest.mark.parametrize("kind,w", [c for c in CASES if c[1] != 1e12])
+@pytest.mark.parametrize("m,n,k", [(2500, 6, 2), (1600, 24, 1), (1300, 40, 24), (900, 60, 33), (800, 100, 2),
+                                   (700, 120, 16)])
+def test_weighted_lstsq_batched(cuda_lib, kind, w, m, n, k):
+    """FP64 items of a batch, beside an ordinary one, and the same requests served by the
+    resident kernel (bitwise the same)."""
+    import paper_0912_2572_gb300 as ts
+    A, B = _problem(m, n, k, kind, w, 10 * n + k)
+    X = _exact(A, B)
+    tol = _tolerance(A, B, X)
+    other = {"A": to_dev(inputs.gaussian(500, 9, 1)), "prec": ts.FP64}
+    for chain_tiles in (2, 16):
+        it = {"A": to_dev(A), "B": to_dev(B), "prec": ts.FP64}
+        (R, Z), _ = ts.batch_solve([it, other], chain_tiles=chain_tiles)
+        R, Z = to_host(R), to_host(Z)
+        err = np.linalg.norm(Z - X) / np.linalg.norm(X)
+        assert err <= tol, (chain_tiles, err, tol)
+        with ts.Server(resident=True, chain_tiles=chain_tiles, ctas_per_sm=1) as srv:
+            _, (Rs, Zs) = srv.submit(it)
+            srv.drain()
+            srv.poll()
+        assert np.array_equal(to_host(Rs), R) and np.array_equal(to_host(Zs), Z)
+
+
+def test_weighted_mixed_items(cuda_lib):
+    """Tree nodes of mixed items: one chain's triangle far above the others'. R carries FP32
+    leaf accuracy by rows of like scale, and X the refinement's."""
+    import paper_0912_2572_gb300 as ts
+    for n in (16, 60, 100):
+        A = inputs.gaussian(6000, n, n)
+        A[:1500] *= 1e6
+        B = inputs.gaussian(6000, 2, n + 1)
+        outs = ts.batch_solve([{"A": to_dev(A), "B": to_dev(B), "prec": ts.MIXED},
+                               {"A": to_dev(A), "prec": ts.MIXED}], chain_tiles=1)
+        X, R = to_host(outs[0][1]), to_host(outs[1][0])
+        assert np.linalg.norm(R - oracle.r_factor(A)) <= 1e-5 * np.linalg.norm(R)
+        Xo = oracle.lstsq(A, B)
+        assert np.linalg.norm(X - Xo) <= 1e-9 * np.linalg.norm(Xo)
