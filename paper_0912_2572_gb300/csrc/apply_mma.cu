@@ -2,16 +2,16 @@
 // (sm_103a): B <- Q^T B, B <- Q B and the thin Q, the same jobs and tiles as the kernels of
 // apply.cu, with the reflectors taken eight at a time in compact-WY form,
 //   H_j..H_j+7 = I - V T V^T,  C <- C - V (T^T (V^T C))   (T for Q),
-// and both products done exactly on 16-bit tensor-core instructions.
+// and both products done on 16-bit tensor-core instructions without rounding inside them.
 //
 // FP64 arithmetic on GB300 is one warp instruction per 64 cycles and SM sub-partition; a
 // 16x8x16 half-precision MMA takes 8. A 64-bit fixed-point number is eight base-256 digits
 // (signed, so adding 0x80..80 makes them its bytes), a half holds a digit exactly, and an
 // FP32 accumulator holds the sum of digit products of equal weight exactly (4 pairs x 256
-// rows x 2^14 = 2^24), so the 43 digit pairs of weight 256^6 and up give a product to 2^-61
-// of ||v|| ||c|| in 43 MMA-shares, 5.4 cycles per entry and product against 64 (the exact
-// splitting of Ozaki, Ogita, Oishi and Rump, 2012). What is left out is below the rounding
-// of the result to its unit, 2^-60 of the column's norm.
+// rows x 2^14 = 2^24), so the 43 digit pairs of weight 256^6 and up take 43 MMA-shares, 5.4
+// cycles per entry and product against 64 (the exact splitting of Ozaki, Ogita, Oishi and
+// Rump, 2012). The 21 pairs left out are below 21 x 2^-21 units of 2^-60 of ||v|| ||c|| a row
+// (24 units in the worst case of 512 rows, signs alike); T is made in FP64.
 //
 // A warp holds 8 columns x up to 144 rows of C in registers: lane 4g + t holds column g,
 // rows 8 b + 2t and 8 b + 2t + 1. That is at once the B fragment of V^T C (its digits are cut
@@ -32,6 +32,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "fixed_point.cuh"
 #include "tsqr_internal.h"
@@ -122,17 +123,79 @@ __device__ __noinline__ double to_double_any(long long x, int sh) {
   return scalbn(__ll2double_rn(x), sh);
 }
 
+// The job from tile q0 (in its order of application) on, from reflector j0 of that tile (mid:
+// the tile is under way), in FP64 with a warp per column: the tile in registers, V from global
+// memory. For tiles of rows that are small beside their column, or reflectors small beside 1,
+// which fixed point would round to a fixed fraction of the column's norm.
+__device__ __noinline__ void apply_rest_fp64(const ApplyParamsT<double> p, const JobDesc job, int q0, int j0, bool mid,
+                                             int c0, int kc) {
+  const int lane = threadIdx.x & 31, n = p.n;
+  for (int c = threadIdx.x >> 5; c < kc; c += blockDim.x >> 5) {
+    double *Bc = p.B + (int64_t)(c0 + c) * p.ldb, *P = Bc + job.piv_row;
+    for (int q = q0; q < job.tile_count; ++q) {
+      const TileDesc td = p.tiles[job.tile_begin + (p.trans ? q : job.tile_count - 1 - q)];
+      const double *Vt = p.V + td.row0;
+      double *Bt = Bc + td.row0;
+      // forming Q there is no input but the pivot block, which is a leaf's first n rows
+      const bool ge = td.kind == GEQRT, zero = p.formq && !(mid && q == q0);
+      double x[16];
+#pragma unroll
+      for (int r = 0; r < 16; ++r) {
+        const int i = lane + 32 * r;
+        x[r] = i < td.nrows && (!zero || (ge && i < n)) ? __ldcg(Bt + i) : 0.0;
+      }
+      const int first = q == q0 ? j0 : p.trans ? 0 : n - 1;
+      for (int j = first; j >= 0 && j < n; j += p.trans ? 1 : -1) {
+        if (p.formq && j > c0 + c) continue;  // reflector j touches columns >= j only
+        int lo, hi;
+        refl_rows(td.kind, j, td.nrows, lo, hi, td.off);
+        const double tau = __ldg(p.tau + td.refl + j), sc = __ldg(p.scl + td.refl + j);
+        const double *Vj = Vt + (int64_t)j * p.ldv;
+        double y[16], a = 0.0, piv = 0.0;
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+          const int i = lane + 32 * r;
+          y[r] = i >= lo && i < hi ? __ldg(Vj + i) : 0.0;
+          a = fma(y[r], x[r], a);
+          if (ge && i == j) piv = x[r];
+        }
+#pragma unroll
+        for (int m = 16; m >= 1; m >>= 1) a += __shfl_xor_sync(kFull, a, m);
+        if (!ge && lane == (j & 31)) piv = __ldcg(P + j);
+        piv = __shfl_sync(kFull, piv, j & 31);
+        const double w = fma(sc, a, piv), np = fma(-tau, w, piv), cf = tau * sc * w;
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+          x[r] = fma(-cf, y[r], x[r]);
+          if (ge && lane + 32 * r == j) x[r] = np;
+        }
+        if (!ge && lane == (j & 31)) P[j] = np;
+      }
+#pragma unroll
+      for (int r = 0; r < 16; ++r)
+        if (lane + 32 * r < td.nrows) Bt[lane + 32 * r] = x[r];
+    }
+  }
+}
+
+// |x| / 2^32, to its bit length
+__device__ __forceinline__ unsigned fx_bits(long long x) {
+  const int h = (int)(x >> 32);
+  return (unsigned)(h ^ (h >> 31));
+}
+
 struct MmaParams {
   ApplyParamsT<double> a;
   int rg, cg;  // row groups and column groups of a CTA's warps
 };
 
 // Shared memory: three buffers of V's digit planes, the pivot block, partial products, T
-// (two), G, column exponents and norms, exchange of the row groups' norms, flags.
+// (two), G, column exponents and norms, exchange of the row groups' norms, counts and lengths,
+// flags, V's light entries, the scales of the pivot block's panels.
 __host__ __device__ inline size_t mma_smem_bytes(int n, int rg, int cg, int nb) {
   const size_t rows = (size_t)16 * nb * rg, kc = 8 * (size_t)cg, np = (size_t)(n + 7) / 8;
   return 3 * 8 * rows * 16 + np * 8 * (kc + 2) * 8 + (size_t)rg * 8 * (kc + 2) * 8 + 2 * 64 * 8 + 64 * 8 +
-         kHelpers * 64 * 8 + kc * 12 + (size_t)rg * kc * 8 + 64;
+         kHelpers * 64 * 8 + kc * 12 + (size_t)rg * kc * 16 + np * kc * 2 + 3 * 8 * 4 + 64;
 }
 
 template <int NB>
@@ -154,8 +217,13 @@ __global__ void __launch_bounds__(384, 1) k_apply_mma(const MmaParams mp) {
   float *nbs = reinterpret_cast<float *>(Es + kc8);
   int *cbad = reinterpret_cast<int *>(nbs + kc8);
   int2 *xn = reinterpret_cast<int2 *>(cbad + kc8);                          // [RG][kc8] exponent, norm
-  int *vbad = reinterpret_cast<int *>(xn + (size_t)RG * kc8);               // [4] by tile: first
+  int2 *xl = xn + (size_t)RG * kc8;                                         // [RG][kc8] counts; bit length
+  int *vbad = reinterpret_cast<int *>(xl + (size_t)RG * kc8);               // [4] by tile: first
                                                                             // reflector not finite
+  int *vlt = vbad + 4;                                                      // [2] step's V is light
+  int *blt = vlt + 2;                                                       // a tile of B is light
+  int *vst = vbad + 8;                                                      // [3][8] V's light entries
+  short *Sc = reinterpret_cast<short *>(vst + 24);  // [NP][kc8]: panel b of Ps is x 2^(60 - E + Sc)
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t = lane & 3;
@@ -189,17 +257,19 @@ __global__ void __launch_bounds__(384, 1) k_apply_mma(const MmaParams mp) {
 
   // V's digits of step s into buffer s mod 3, a row and two reflectors per thread and turn: v =
   // scale * tail in units of 2^-61, 1 on a leaf tile's diagonal, 0 above it. A thread's
-  // entries of kTurns turns are loaded together.
-  constexpr int kTurns = 6;
+  // entries of kTurns turns are loaded together, a round ahead (six turns in one round were
+  // a tenth of the kernel's code, which its loop streams through the instruction cache).
+  constexpr int kTurns = 2;
   auto cut_v = [&](int s, int id, int count) {
     const TileDesc td = tile_at(s);
     const int b = panel_at(s);
     unsigned char *buf = smraw + (size_t)(s % 3) * 8 * plane_bytes;
-    for (int e0 = id; e0 < 4 * rows; e0 += kTurns * count) {
-      double x[kTurns][2], sc[2];
-      const int h = e0 & 3;  // count is a multiple of 4: the same reflectors every turn
+    int light[2] = {0, 0};  // light entries of a reflector
+    const int h = id & 3;  // count is a multiple of 4: the same reflectors every turn
+    double sc[2], xn2[kTurns][2];
 #pragma unroll
-      for (int q = 0; q < 2; ++q) sc[q] = 8 * b + 2 * h + q < n ? __ldg(p.scl + td.refl + 8 * b + 2 * h + q) : 0.0;
+    for (int q = 0; q < 2; ++q) sc[q] = 8 * b + 2 * h + q < n ? __ldg(p.scl + td.refl + 8 * b + 2 * h + q) : 0.0;
+    auto load = [&](int e0) {
 #pragma unroll
       for (int k = 0; k < kTurns; ++k)
 #pragma unroll
@@ -207,8 +277,18 @@ __global__ void __launch_bounds__(384, 1) k_apply_mma(const MmaParams mp) {
           const int r = (e0 + k * count) >> 2, j = 8 * b + 2 * h + q;
           int lo, hi;
           refl_rows(td.kind, j, td.nrows, lo, hi, td.off);
-          x[k][q] = (j < n && r >= lo && r < hi) ? __ldg(p.V + td.row0 + r + (int64_t)j * p.ldv) : 0.0;
+          xn2[k][q] = (j < n && r >= lo && r < hi) ? __ldg(p.V + td.row0 + r + (int64_t)j * p.ldv) : 0.0;
         }
+    };
+    load(id);
+#pragma unroll 1
+    for (int e0 = id; e0 < 4 * rows; e0 += kTurns * count) {
+      double x[kTurns][2];
+#pragma unroll
+      for (int k = 0; k < kTurns; ++k)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) x[k][q] = xn2[k][q];
+      load(e0 + kTurns * count);
 #pragma unroll
       for (int k = 0; k < kTurns; ++k) {
         const int r = (e0 + k * count) >> 2;
@@ -220,13 +300,23 @@ __global__ void __launch_bounds__(384, 1) k_apply_mma(const MmaParams mp) {
           const double z = x[k][q] * sc[q];
           w[q] = (td.kind == GEQRT && r == j && j < n) ? 1ll << 61 : fx_of_double(__double_as_longlong(z), 61);
           // |v| <= 1 but for rounding; anything else is not a reflector
-          if ((unsigned)(__double2hiint(z) & 0x7fffffff) > (1023u << 20 | 0x80000u)) atomicMin(vbad + ((s / NP) & 3), j);
+          const unsigned hz = (unsigned)__double2hiint(z) & 0x7fffffffu;
+          if (hz > (1023u << 20 | 0x80000u)) atomicMin(vbad + ((s / NP) & 3), j);
+          if (hz - 1u < ((1023u - kFxLightBits) << 20)) ++light[q];
         }
         uint32_t d[8];
         digits2(w[0], w[1], d);
         unsigned char *dst = buf + (size_t)r * 16 + 4 * h;
 #pragma unroll
         for (int i = 0; i < 8; ++i) *reinterpret_cast<uint32_t *>(dst + (size_t)i * plane_bytes) = d[i];
+      }
+    }
+    if (!p.trans) {  // (a warp's lanes take the same turns)
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+#pragma unroll
+        for (int m = 4; m <= 16; m <<= 1) light[q] += __shfl_xor_sync(kFull, light[q], m);
+        if (lane < 4 && light[q] > 0) atomicAdd(vst + (s % 3) * 8 + 2 * lane + q, light[q]);
       }
     }
   };
@@ -261,6 +351,20 @@ __global__ void __launch_bounds__(384, 1) k_apply_mma(const MmaParams mp) {
     const TileDesc td = tile_at(s);
     const int b = panel_at(s);
     const double tl = (lane < 8 && 8 * b + lane < n) ? __ldg(p.tau + td.refl + 8 * b + lane) : 0.0;
+    if (!p.trans) {
+      // light: a quarter of a reflector's entries, or all of them (its column of Q falls off
+      // along the rows as A's does; one to three rows may be small by chance)
+      bool light = false;
+      if (lane < 8) {
+        const int l = vst[(s % 3) * 8 + lane];
+        int lo, hi;
+        refl_rows(td.kind, 8 * b + lane, td.nrows, lo, hi, td.off);
+        light = l > 0 && td.off == 0 && (4 * (l - 4) > hi - lo || (l == hi - lo && (td.kind != TSQRT || l > 3)));
+        vst[(s % 3) * 8 + lane] = 0;
+      }
+      light = __any_sync(kFull, light);
+      if (lane == 0) vlt[s & 1] = light;
+    }
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
       const int i = lane + 32 * e;
@@ -293,6 +397,9 @@ __global__ void __launch_bounds__(384, 1) k_apply_mma(const MmaParams mp) {
   };
 
   if (tid < 4) vbad[tid] = n;
+  if (tid < 3) vlt[tid] = 0;  // and blt
+  if (tid < 24) vst[tid] = 0;
+  for (int e = tid; e < NP * kc8; e += blockDim.x) Sc[e] = 0;
   for (int c = tid; c < kc8; c += blockDim.x) {
     Es[c] = kFxNone;
     nbs[c] = 0.f;
@@ -319,8 +426,26 @@ __global__ void __launch_bounds__(384, 1) k_apply_mma(const MmaParams mp) {
       sq += __shfl_xor_sync(kFull, sq, 1);
       sq += __shfl_xor_sync(kFull, sq, 2);
       if (e != 0 && fin) fx_grow(E, nb, (int)e - 1022, sq);
-      if (E != kFxNone)
+      if (!p.trans && E != kFxNone)
         for (int i = t; i < n; i += 4) Ps[i * kcp + col] = fx_of_double(__double_as_longlong(__ldcg(Bc + pr + i)), 60 - E);
+      // forward, each panel at its own scale, its largest entry below 2^56
+      for (int b = 0; p.trans && b < NP; ++b) {
+        long long x[2];
+        int eb = 0;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const int i = 8 * b + t + 4 * q;
+          x[q] = E != kFxNone && cin && i < n ? __double_as_longlong(__ldcg(Bc + pr + i)) : 0;
+          eb = max(eb, (int)((x[q] >> 52) & 0x7ff));
+        }
+        eb = max(eb, __shfl_xor_sync(kFull, eb, 1));
+        eb = max(eb, __shfl_xor_sync(kFull, eb, 2));
+        const int sc = eb == 0 ? 0 : min(max(E - (eb - 1022) - 4, 0), 400);
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+          if (8 * b + t + 4 * q < n) Ps[(8 * b + t + 4 * q) * kcp + col] = fx_of_double(x[q], 60 - E + sc);
+        if (t == 0) Sc[b * kc8 + col] = (short)sc;
+      }
       if (t == 0) {
         Es[col] = E;
         nbs[col] = nb;
@@ -337,7 +462,42 @@ __global__ void __launch_bounds__(384, 1) k_apply_mma(const MmaParams mp) {
   __syncthreads();
 
   long long v[4 * NB];
-  for (int s = 0; s < S; ++s) {
+  int cur = 0;   // this lane's column of the tile is x 2^(60 - E + cur)
+  int ttop = 0;  // bit length of the tile's entries at its start, above 32
+  int pdom = -1; // the last panel of the pivot block found not short in this tile
+  auto store_tile = [&](const TileDesc &td) {
+    const int E = Es[col];
+    const int sh = (E == kFxNone ? 0 : E) - 60 - cur, ht = td.nrows;
+    const bool bad = cbad[col] != 0, wide = sh < -900 || sh > 900;
+    double *dst = Bc + td.row0;
+    const bool al = (reinterpret_cast<uintptr_t>(dst) & 15) == 0;
+    const int beg = td.kind == GEQRT && p.trans ? n : 0;
+#pragma unroll
+    for (int q = 0; q < 2 * NB; ++q) {
+      const int i = 16 * NB * rg + 2 * t + 8 * q;
+      if (beg > 0) {  // the pivot block leaves the leaf tile
+        if (i < n) Ps[i * kcp + col] = v[2 * q];
+        if (i + 1 < n) Ps[(i + 1) * kcp + col] = v[2 * q + 1];
+      }
+      double2 d;
+      if (wide)
+        d = make_double2(to_double_any(v[2 * q], sh), to_double_any(v[2 * q + 1], sh));
+      else
+        d = make_double2(fx_to_double(v[2 * q], sh), fx_to_double(v[2 * q + 1], sh));
+      if (bad) d.x = d.y = __longlong_as_double(0x7ff8000000000000ll);
+      if (cin && al && i >= beg && i + 1 < ht) {
+        *reinterpret_cast<double2 *>(dst + i) = d;
+      } else if (cin) {
+        if (i >= beg && i < ht) dst[i] = d.x;
+        if (i + 1 >= beg && i + 1 < ht) dst[i + 1] = d.y;
+      }
+    }
+  };
+  int s = 0;
+  // the rest of the job goes on in FP64 when a step's V is light (from that step on) or a tile of
+  // B is (from the tile on); both are the same for the whole CTA
+  for (; s < S; ++s) {
+    if (vlt[s & 1]) break;
     const TileDesc td = tile_at(s);
     const int pi = s % NP, b = panel_at(s);
     const int ht = td.nrows;
@@ -352,7 +512,9 @@ __global__ void __launch_bounds__(384, 1) k_apply_mma(const MmaParams mp) {
         else if (s + 2 < S) cut_v(s + 2, tid - MT - 32, 32 * (kHelpers - 1));
       }
     } else {
+      bool skip = false;
       if (pi == 0) {  // a new tile: its rows, exponents, integers
+        cur = 0;
         if (p.formq) {
 #pragma unroll
           for (int r = 0; r < 4 * NB; ++r) v[r] = 0;
@@ -395,10 +557,51 @@ __global__ void __launch_bounds__(384, 1) k_apply_mma(const MmaParams mp) {
             if (x.x == 2047) bad = true;
             else if (x.x != 0) fx_grow(E, nb, x.x - 1022, __int_as_float(x.y));
           }
+          {
+            // light entries are counted in leaves and nodes; under a chain's triangle heavy rows
+            // mix with light pivot rows in FP64 too
+            if (td.kind != TSQRT) {
+              const int lim = (E + 1023 - kFxLightBits) * (1 << 20);
+              unsigned cnt = 0;
+#pragma unroll
+              for (int r = 0; r < 4 * NB; ++r) {
+                const unsigned h = (unsigned)(v[r] >> 32) & 0x7fffffffu;
+                if (h != 0) cnt += (int)h < lim ? 0x10001u : 1u;
+              }
+              cnt += __shfl_xor_sync(kFull, cnt, 1);
+              cnt += __shfl_xor_sync(kFull, cnt, 2);
+              if (t == 0) xl[rg * kc8 + col].x = (int)cnt;
+            }
+            const int sh = 60 - (E == kFxNone ? 0 : E);
+#pragma unroll
+            for (int r = 0; r < 4 * NB; ++r) v[r] = fx_of_double(v[r], sh);
+          }
           bar_main(MT);  // the old exponents have been read
+          int te = -100000;  // the tile's entries are below 2^(E + te)
+          for (int r = 0; r < RG; ++r) {
+            const int x = xn[r * kc8 + col].x;
+            if (x != 0) te = max(te, x - 1022 - E);
+          }
+          ttop = 28 + te;
+          // (a TSQRT tile with an entry above 2^(E - 7) is not light: 512 rows)
+          if (te > -100000 && !bad && (td.kind != TSQRT || te < -6)) {
+            unsigned cnt = td.kind == TSQRT ? (unsigned)ht : 0;
+            float sum = 0.f;
+            for (int r = 0; r < RG; ++r) {
+              const int2 x = xn[r * kc8 + col];
+              if (td.kind != TSQRT) cnt += (unsigned)xl[r * kc8 + col].x;
+              if (x.x != 0) sum += __int_as_float(x.y) * exp2f((float)max(2 * (x.x - 1022 - E), -100));
+            }
+            if (td.off == 0 && fx_light(cnt & 0xffff, cnt >> 16, sum, 0, td.kind == TTQRT)) *blt = 1;
+          }
           if (rg == 0) {
-            if (E != E0 && E0 != kFxNone)
-              for (int i = t; i < n; i += 4) Ps[i * kcp + col] = fx_shift(Ps[i * kcp + col], E0 - E);
+            if (E != E0 && E0 != kFxNone) {
+              if (p.trans) {  // the panels' scales are relative to the exponent
+                for (int b2 = t; b2 < NP; b2 += 4) Sc[b2 * kc8 + col] = (short)min(Sc[b2 * kc8 + col] + E - E0, 30000);
+              } else {
+                for (int i = t; i < n; i += 4) Ps[i * kcp + col] = fx_shift(Ps[i * kcp + col], E0 - E);
+              }
+            }
             if (t == 0) {
               Es[col] = E;
               nbs[col] = nb;
@@ -406,10 +609,8 @@ __global__ void __launch_bounds__(384, 1) k_apply_mma(const MmaParams mp) {
             }
             __syncwarp();
           }
-          const int sh = 60 - (E == kFxNone ? 0 : E);
-#pragma unroll
-          for (int r = 0; r < 4 * NB; ++r) v[r] = fx_of_double(v[r], sh);
-          if (ge && !p.trans) bar_main(MT);
+          bar_main(MT);
+          skip = *blt != 0;  // light: the rest in FP64
         }
         if (ge && !p.trans) {  // the pivot block moves into the leaf tile
 #pragma unroll
@@ -423,7 +624,49 @@ __global__ void __launch_bounds__(384, 1) k_apply_mma(const MmaParams mp) {
       }
       const uint32_t pl = smem_addr(smraw) + (uint32_t)(s % 3) * 8 * plane_bytes + (uint32_t)(16 * NB * rg) * 16u;
       // forming the thin Q, reflector j touches columns >= j only
-      const bool act = !p.formq || (c0 >> 3) + cg >= b;
+      const bool act = !skip && (!p.formq || (c0 >> 3) + cg >= b);
+      // Forward, a column whose remainder (the panels of the pivot block from b on, the tile)
+      // has become short is shifted up to fill its bits again, as in the factorization: where
+      // R is ill-conditioned the components of Q^T B fall off like R's rows, and R^-1 magnifies
+      // what they lost (X of consistent systems of 4M x 64 at condition number 1e4 by Q^T B and the
+      // solve 8.9e-15, with it 3.2e-15, in FP64 2.8e-15). Entries of the remainder stay below
+      // 2^55, its norm below 2^60.
+      if (p.trans && act) {
+        int top = ttop;  // the tile's entries are below 2^(32 + top)
+        if (pi != 0) {
+          unsigned len = 0;
+          for (int r = 0; r < RG; ++r) len |= (unsigned)xl[r * kc8 + col].y;
+          top = 32 - __clz((int)len);
+        } else {
+          pdom = -1;
+        }
+        // the pivot block's panels from b on, the last first: on long chains they are far above the
+        // tile, and while one that is not short is to come the column stays as it is
+        bool look = top < 21 && b > pdom;
+        for (int b2 = ge ? b - 1 : NP - 1; b2 >= b && __any_sync(kFull, look); --b2) {
+          int pt = -100000;
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            const int i = 8 * b2 + t + 4 * q;
+            const long long x = i < n ? Ps[i * kcp + col] : 0;
+            if (x != 0) pt = max(pt, 32 - __clz((int)fx_bits(x)) + cur - Sc[b2 * kc8 + col]);
+          }
+          pt = max(pt, __shfl_xor_sync(kFull, pt, 1));
+          pt = max(pt, __shfl_xor_sync(kFull, pt, 2));
+          top = max(top, pt);
+          if (look && pt >= 21) pdom = b2, look = false;
+        }
+        if (__any_sync(kFull, look)) {
+          const int d = look ? min(23 - top, 23) : 0;
+          cur += d;
+#pragma unroll
+          for (int q = 0; q < 2 * NB; ++q)
+            if (!ge || 16 * NB * rg + 8 * q >= 8 * b) {
+              v[2 * q] = (long long)((unsigned long long)v[2 * q] << d);
+              v[2 * q + 1] = (long long)((unsigned long long)v[2 * q + 1] << d);
+            }
+        }
+      }
       if (act) {
         float acc[9][4];
 #pragma unroll
@@ -444,10 +687,17 @@ __global__ void __launch_bounds__(384, 1) k_apply_mma(const MmaParams mp) {
           }
         }
         longlong2 w = make_longlong2(combine_w(acc, 0), combine_w(acc, 1));  // reflector g, columns 2t, 2t+1
+        const int cu0 = __shfl_sync(kFull, cur, 8 * t), cu1 = __shfl_sync(kFull, cur, 8 * t + 4);  // of columns 2t, 2t+1
         if (rg == 0 && !ge) {
           const longlong2 q = *reinterpret_cast<const longlong2 *>(Ps + (8 * b + g) * kcp + 8 * cg + 2 * t);
+          const short *sc = Sc + b * kc8 + 8 * cg + 2 * t;
+          const int d0 = cu0 - sc[0], d1 = cu1 - sc[1];
           w.x += q.x;
           w.y += q.y;
+          if (__any_sync(kFull, d0 != 0 || d1 != 0)) {
+            w.x += fx_shift(q.x, d0) - q.x;
+            w.y += fx_shift(q.y, d1) - q.y;
+          }
         }
         *reinterpret_cast<longlong2 *>(Wp + (rg * 8 + g) * kcp + 8 * cg + 2 * t) = w;
       }
@@ -472,6 +722,13 @@ __global__ void __launch_bounds__(384, 1) k_apply_mma(const MmaParams mp) {
         const long long y0 = -((h0 << 1) + (m0 >> 29)), y1 = -((h1 << 1) + (m1 >> 29));
         if (rg == 0 && !ge) {
           long long *P = Ps + (8 * b + 2 * t) * kcp + col;
+          const int d = cur - Sc[b * kc8 + col];
+          if (__any_sync(kFull, d != 0)) {
+            P[0] = fx_shift(P[0], d);
+            P[kcp] = fx_shift(P[kcp], d);
+            __syncwarp();
+            if (t == 0) Sc[b * kc8 + col] = (short)cur;
+          }
           P[0] += y0;
           P[kcp] += y1;
         }
@@ -516,49 +773,48 @@ __global__ void __launch_bounds__(384, 1) k_apply_mma(const MmaParams mp) {
             v[2 * q + e] = c;
           }
         }
+        if (p.trans && __any_sync(kFull, b >= pdom)) {
+          // of what remains of the column: a sample of its rows, all of them if those are short
+          unsigned len = 0;
+          auto all = [&](auto step) {
+#pragma unroll
+            for (int q = 0; q < 2 * NB; q += decltype(step)::value)
+              if (!ge || 16 * NB * rg + 8 * q > 8 * b) len |= fx_bits(v[2 * q]) | fx_bits(v[2 * q + 1]);
+            len |= __shfl_xor_sync(kFull, len, 1);
+            len |= __shfl_xor_sync(kFull, len, 2);
+          };
+          all(std::integral_constant<int, 4>());
+          if (__any_sync(kFull, len < (1u << 20))) all(std::integral_constant<int, 1>());
+          if (t == 0) xl[rg * kc8 + col].y = (int)len;
+        }
+        if (p.trans && ge && rg == 0 && t == 0) Sc[b * kc8 + col] = (short)cur;  // a leaf's rows of the pivot block
       }
-      if (pi == NP - 1) {  // the tile is done
-        const int E = Es[col];
-        const int sh = (E == kFxNone ? 0 : E) - 60;
+      if (pi == NP - 1 && !skip) {  // the tile is done
         // a reflector that is not finite spoils the columns it touches
         if (vbad[(s / NP) & 3] < (p.formq ? min(n, c0 + col + 1) : n) && t == 0 && rg == 0) cbad[col] = 1;
         if (RG > 1) bar_main(MT);
         else __syncwarp();
-        const bool bad = cbad[col] != 0, wide = sh < -900 || sh > 900;
-        double *dst = Bc + r0;
-        const bool al = (reinterpret_cast<uintptr_t>(dst) & 15) == 0;
-        const int beg = ge && p.trans ? n : 0;
-#pragma unroll
-        for (int q = 0; q < 2 * NB; ++q) {
-          const int i = rbase + 8 * q;
-          if (beg > 0) {  // the pivot block leaves the leaf tile
-            if (i < n) Ps[i * kcp + col] = v[2 * q];
-            if (i + 1 < n) Ps[(i + 1) * kcp + col] = v[2 * q + 1];
-          }
-          double2 d;
-          if (wide)
-            d = make_double2(to_double_any(v[2 * q], sh), to_double_any(v[2 * q + 1], sh));
-          else
-            d = make_double2(fx_to_double(v[2 * q], sh), fx_to_double(v[2 * q + 1], sh));
-          if (bad) d.x = d.y = __longlong_as_double(0x7ff8000000000000ll);
-          if (cin && al && i >= beg && i + 1 < ht) {
-            *reinterpret_cast<double2 *>(dst + i) = d;
-          } else if (cin) {
-            if (i >= beg && i < ht) dst[i] = d.x;
-            if (i + 1 >= beg && i + 1 < ht) dst[i + 1] = d.y;
-          }
-        }
+        store_tile(td);
       }
     }
     __syncthreads();
+    if (*blt) break;
   }
-  // the pivot block, unless the last tile held it (a leaf, backward)
-  if (!helper && rg == 0 && cin && !(!p.trans && tile_at(S - 1).kind == GEQRT)) {
+  const bool rest = s < S, mid = rest && s % NP != 0;
+  if (mid && !helper) store_tile(tile_at(s));
+  // the pivot block, unless it has not changed, or a leaf tile holds it (backward, the last one or
+  // one under way)
+  const bool in_leaf = !p.trans && (!rest || mid) && tile_at(rest ? s : S - 1).kind == GEQRT;
+  if (!helper && rg == 0 && cin && s > 0 && !in_leaf) {
     const int E = Es[col];
-    const int sh = (E == kFxNone ? 0 : E) - 60;
     const bool bad = cbad[col] != 0;
     for (int i = t; i < n; i += 4)
-      Bc[pr + i] = bad ? __longlong_as_double(0x7ff8000000000000ll) : to_double_any(Ps[i * kcp + col], sh);
+      Bc[pr + i] = bad ? __longlong_as_double(0x7ff8000000000000ll)
+                       : to_double_any(Ps[i * kcp + col], (E == kFxNone ? 0 : E) - 60 - Sc[(i >> 3) * kc8 + col]);
+  }
+  if (rest) {
+    __syncthreads();
+    apply_rest_fp64(p, job, s / NP, p.trans ? 0 : min(n, 8 * panel_at(s) + 8) - 1, mid, c0, kc);
   }
 }
 

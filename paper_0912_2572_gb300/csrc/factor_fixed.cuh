@@ -112,25 +112,6 @@ __device__ __forceinline__ FxRefl fx_reflector(long long alpha, unsigned __int12
   return f;
 }
 
-// Light tiles. An entry of 2^-s of its column's norm keeps 60 - s bits here, where FP64 keeps
-// 53 of every entry, and what it lost matters once the heavy rows of the column are eliminated:
-// in weighted least squares with the heavy rows first (weights of 1e8 are ordinary for soft
-// constraints) the light rows alone determine the rest of the unknowns. A tile is light in a
-// column, and its job goes on in FP64 from there, if the root mean square of the tile's nonzero
-// entries is below 2^-12 of 2^E, or more of them than a smooth distribution would have (its
-// density at zero is below 1 / rms: eight times that) are below 2^-16. The rows of a chain of
-// M alike rows are at 2^-(1 + log2(M) / 2), so plain chains of up to 2^22 rows stay. A node's
-// triangle falls off along its rows by itself when A is ill-conditioned: there a quarter of the
-// entries may be that small, and the later pieces of a triangle are not looked at. Costs two
-// instructions per entry and tile, beside 37 cycles per entry and step.
-constexpr int kFxLightBits = 16;
-// nz entries, nl of them light, their squares' sum sq 4^d in units of the column's 4^E
-__device__ __forceinline__ bool fx_light(unsigned nz, unsigned nl, float sq, int d, bool tri) {
-  if (nz == 0) return false;
-  const float fz = (float)nz, q = sq * exp2f((float)max(2 * d, -100)) / fz;
-  return q < 0x1p-24f || (float)nl > 4.f + fz * fmaxf(0x1p-13f * rsqrtf(q), tri ? 0.25f : 0.f);
-}
-
 // Shared memory of the job: tails of two reflectors, the next pivot column, scalars (two
 // steps' limbs; every reflector's for the tile's end), column exponents and norms, R and the
 // scales of its row blocks.

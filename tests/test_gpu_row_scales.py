@@ -123,3 +123,99 @@ def test_weighted_mixed_items(cuda_lib):
         assert np.linalg.norm(R - oracle.r_factor(A)) <= 1e-5 * np.linalg.norm(R)
         Xo = oracle.lstsq(A, B)
         assert np.linalg.norm(X - Xo) <= 1e-9 * np.linalg.norm(Xo)
+
+
+@pytest.mark.parametrize("kind,w", [c for c in CASES if c[1] != 1e12])
+@pytest.mark.parametrize("m,n,k", [(900, 24, 12), (1300, 40, 24), (1500, 8, 40)])
+def test_weighted_qt_b_then_solve(cuda_lib, kind, w, m, n, k):
+    """Q^T B of more than 8 columns and the triangular solve, and the same through CAQR
+    (whose trailing update is a Q^T B)."""
+    import paper_0912_2572_gb300 as ts
+    A, B = _problem(m, n, k, kind, w, 10 * n + k)
+    X = _exact(A, B)
+    tol = _tolerance(A, B, X)
+    for how in ("chain", "tree", "caqr"):
+        Ad = to_dev(A)
+        if how == "caqr":
+            F = ts.caqr(Ad, panel=(n + 1) // 2)
+        else:
+            F = ts.factor(Ad, arity=0 if how == "chain" else 2, two_level=how == "chain")
+        Z = to_host(F.solve_r(F.apply_qt(to_dev(B))))
+        F.free()
+        err = np.linalg.norm(Z - X) / np.linalg.norm(X)
+        assert err <= tol, (how, err, tol)
+
+
+@pytest.mark.parametrize("m,n,two", [(900, 24, True), (1300, 40, False), (700, 100, True)])
+def test_light_rows_of_q(cuda_lib, m, n, two):
+    """Rows of Q far below their column keep their digits as rows: three rows weighted by
+    1e12, the other rows of Q's first three columns are 1e-12 of them; and Q Q^T B = B for a
+    B of such rows, by rows."""
+    import paper_0912_2572_gb300 as ts
+    A, B = _problem(m, n, 24, "dense", 1e12, n)
+    F = ts.factor(to_dev(A), two_level=two)
+    Q = to_host(F.form_q())
+    Z = to_host(F.apply_q(F.apply_qt(to_dev(B))))
+    F.free()
+    Qo = oracle.qr(A)[0]
+    assert np.linalg.norm((Q - Qo)[3:, :3]) <= 1e-12 * np.linalg.norm(Qo[3:, :3])
+    assert np.linalg.norm((Q - Qo)[:, 3:]) <= 1e-12 * np.sqrt(n)
+    assert oracle.orth_error(Q) <= 1e-13
+    assert np.linalg.norm((Z - B)[3:]) <= 1e-12 * np.linalg.norm(B[3:])
+
+
+@pytest.mark.parametrize("m,n,k,decades", [(1_000_000, 64, 32, 4.0), (4_000_000, 32, 16, 6.0)])
+def test_small_components_of_tall_qt_b(cuda_lib, m, n, k, decades):
+    """The same on tall matrices, where a tile is a small part of its column: consistent
+    systems with exactly representable right-hand sides (A rounded to 2^-30, X small whole
+    numbers), within 2.5 times the FP64 kernel's error."""
+    import torch
+    import paper_0912_2572_gb300 as ts
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    V = torch.linalg.qr(torch.randn((n, n), generator=g, dtype=torch.float64, device="cuda"))[0]
+    s = 10.0 ** (-decades * torch.arange(n, dtype=torch.float64, device="cuda") / (n - 1))
+    A = torch.randn((m, n), generator=g, dtype=torch.float64, device="cuda") @ (V * s).T
+    A = ts.colmajor((A * 2.0 ** 30).round() / 2.0 ** 30)
+    X = torch.randint(-8, 9, (n, k), generator=g, device="cuda").double()
+    B = A @ X
+    F = ts.factor(A, leaf_h=512)
+    at_once = F.solve_r(F.apply_qt(ts.colmajor(B.clone())))
+    eights = torch.cat([F.solve_r(F.apply_qt(ts.colmajor(B[:, c:c + 8].clone()))) for c in range(0, k, 8)], 1)
+    F.free()
+    assert float((at_once - X).norm()) <= 2.5 * float((eights - X).norm())
+
+
+@pytest.mark.parametrize("k", [9, 16, 32])
+@pytest.mark.parametrize("decades", [4.0, 6.0])
+def test_small_components_of_qt_b(cuda_lib, decades, k):
+    """B in the range of an ill-conditioned A: the components of Q^T B fall off like R's rows and
+    R^-1 magnifies their errors. X through Q^T B of all columns at once is as near the exact
+    solution (FP64 refined with residuals in extended precision) as eight columns at a time
+    on the FP64 kernel, within a factor of two; so is X through CAQR."""
+    import paper_0912_2572_gb300 as ts
+    m, n = 20000, 32
+    A = inputs.graded(m, n, decades, seed_g=int(decades) + k, seed_v=2)
+    B = A @ inputs.gaussian(n, k, 3) + 1e-6 * inputs.gaussian(m, k, 4)
+    Q, R = oracle.qr(A)[:2]
+    X = np.zeros((n, k), np.longdouble)
+    for _ in range(6):
+        r = (B - A.astype(np.longdouble) @ X).astype(np.float64)
+        X = X + np.linalg.solve(R, Q.T @ r)
+
+    def err(Z):
+        return float(np.linalg.norm(to_host(Z) - X) / np.linalg.norm(X))
+
+    Ad, Bd = to_dev(A), to_dev(B)
+    F = ts.factor(Ad, leaf_h=144)
+    at_once = err(F.solve_r(F.apply_qt(to_dev(B))))
+    by_eights = []
+    for c in range(0, k, 8):
+        by_eights.append(to_host(F.solve_r(F.apply_qt(to_dev(B[:, c:c + 8])))))
+    F.free()
+    e8 = err(to_dev(np.concatenate(by_eights, axis=1)))
+    Fc = ts.caqr(Ad, panel=16)
+    ec = err(Fc.solve_r(Fc.apply_qt(Bd)))
+    Fc.free()
+    print(f"at once {at_once:.2e}, by eights {e8:.2e}, caqr {ec:.2e}")
+    assert at_once <= 2 * e8 and ec <= 2 * e8, (at_once, e8, ec)
