@@ -589,7 +589,7 @@ static tsqr_status run_factor(tsqr_factors *F, const double *A, int64_t lda, dou
 // Launch li of the plan applied to B's columns [c0, c0 + kg) (kg <= 64; the warp kernel
 // for kg <= 8): Q^T in forward launch order, Q in reverse.
 static tsqr_status apply_launch(const tsqr_factors *F, double *B, int64_t ldb, int c0, int kg, int trans, int formq,
-                                int li, cudaStream_t s) {
+                                int li, cudaStream_t s, int mma_min = 9) {
   const Plan &pl = F->plan();
   ApplyParams p{};
   p.V = F->V;
@@ -621,7 +621,7 @@ static tsqr_status apply_launch(const tsqr_factors *F, double *B, int64_t ldb, i
     CUDA_TRY(launch_apply_tile(p, ld.job_count, s));
     return TSQR_OK;
   }
-  if (kg > 8) {
+  if (kg >= mma_min) {
     CUDA_TRY(launch_apply_mma(p, ld.job_count, li == 0 ? pl.tile_h : pl.n, narrow ? 16 : 64, s));
     return TSQR_OK;
   }
@@ -640,15 +640,16 @@ static int apply_group(int k) { return (k <= 8) ? 8 : 64; }
 // against 9.4), wider ones 64 columns at a time on the tensor cores.
 static int formq_group(int n) { return (n <= 8) ? 4 : 64; }
 
+// mma_min: the fewest columns that go to the tensor-core kernel.
 static tsqr_status run_apply(const tsqr_factors *F, double *B, int64_t ldb, int k, int trans, int formq,
-                             cudaStream_t s, int group = 0) {
+                             cudaStream_t s, int mma_min = 9) {
   const Plan &pl = F->plan();
   const int nl = (int)pl.launches.size();
-  if (group == 0) group = formq ? formq_group(k) : apply_group(k);
+  const int group = formq ? formq_group(k) : apply_group(k);
   for (int c0 = 0; c0 < k; c0 += group) {
     const int kg = std::min(group, k - c0);
     for (int q = 0; q < nl; ++q) {
-      tsqr_status st = apply_launch(F, B, ldb, c0, kg, trans, formq, trans ? q : nl - 1 - q, s);
+      tsqr_status st = apply_launch(F, B, ldb, c0, kg, trans, formq, trans ? q : nl - 1 - q, s, mma_min);
       if (st != TSQR_OK) return st;
     }
   }
@@ -1921,10 +1922,12 @@ tsqr_status tsqr_lstsq(const double *A, int64_t m, int32_t n, int64_t lda, const
   int32_t *status = nullptr;
   // B's columns are factored along unless they take A's over the edge of the eight-warp job
   // (64 columns, two CTAs per SM) and there are enough rows for a separate pass of Q^T B to cost
-  // less than the sixteen-warp job does: x 64 with 1 / 4 / 8 right-hand sides, 1,000 rows 1.46 /
-  // 2.01 / 2.68 ms against 1.31 fused, 30,000 2.10 / 2.69 / 3.44 against 2.14, 300,000 4.89 /
-  // 5.88 / 7.09 against 6.75, 1M 9.8 / 11.9 / 14.9 against 15.1
-  const bool fused = (n + k) <= 64 || (n + k <= 128 && (n > 64 || m <= (int64_t)24000 * k));
+  // less than the sixteen-warp job does. Fused against a pass of its own, x 64: with 1 column
+  // 30,000 rows 2.14 ms against 2.10 and 300,000 6.75 against 4.89; on the tensor cores (from 5
+  // columns) 8 columns 5,000 rows 1.80 against 1.85, 15,000 2.08 / 1.84, 300,000 6.9 / 5.1, 1M
+  // 14.8 / 11.4; 16 columns 2,000 rows 1.49 / 1.55, 30,000 2.11 / 1.97; 64 columns 30,000 2.98 /
+  // 2.04, 1M 25.9 / 14.6
+  const bool fused = (n + k) <= 64 || (n + k <= 128 && (n > 64 || m <= (k < 5 ? (int64_t)24000 * k : 20000)));
   st = get_plan(m, n, fused ? n + k : n, leaf_h, arity, flags, f->dp);
   if (st == TSQR_OK) st = factors_alloc(f, s);
   if (st == TSQR_OK) {
@@ -1946,9 +1949,9 @@ tsqr_status tsqr_lstsq(const double *A, int64_t m, int32_t n, int64_t lda, const
       st = run_factor(f, A, lda, W, m, s);  // Q^T B computed with the factorization
     } else {
       st = run_factor(f, A, lda, nullptr, 0, s);
-      // eight columns at a time (FP64): the small components of Q^T B keep their bits, which
-      // an ill-conditioned R^{-1} magnifies
-      if (st == TSQR_OK) st = run_apply(f, W, m, k, 1, 0, s, 8);
+      // from 5 columns on the tensor cores (n > 56 here: the warp kernel takes 7.1 ms for 300,000 x
+      // 64 with 8, this one 5.1; with 4 columns 1M x 64 12.2 and 12.0)
+      if (st == TSQR_OK) st = run_apply(f, W, m, k, 1, 0, s, 5);
     }
   }
   if (st == TSQR_OK) {
