@@ -7,7 +7,7 @@
 // everything in reverse.
 //
 // B with at most 8 columns runs here, and the thin Q of up to 8 columns in passes of 4, and 9
-// to 16 columns against few reflectors (k_apply_tile); other widths go to the tensor-core
+// to 32 columns against few reflectors (k_apply_tile); other widths go to the tensor-core
 // kernel (apply_mma.cu). k_apply_warp: one warp per job; each
 // reflector is a dot product over the tile rows, one warp-level transpose-reduce, and an
 // update; no block barrier is needed. With 4 columns a job stages 16.6 KB of a 512-row tile,
@@ -395,23 +395,23 @@ __global__ void __launch_bounds__(128, 3) k_apply_vec(const ApplyParamsT<double>
   for (int j = lane; j < n; j += 32) B[pr + j] = Pf[j];
 }
 
-// ------------------------------------------- 9..16 columns, few reflectors: a CTA per job
+// ------------------------------------------- 9..32 columns, few reflectors: a CTA per job
 // With few reflectors per tile the tensor-core kernel is bound by what it does once per tile
 // and panel (digits of V and of the tile, eight of its warps on two column groups); here the
-// tile of up to 16 columns is in shared memory, a half-warp per column, and the next
+// tile of up to 32 columns is in shared memory, a half-warp per column of 16, and the next
 // reflector's tail and pivot row are loaded one step ahead. The columns rotate over the
 // warps with the reflector, so that no SM sub-partition's FP64 pipe takes the extra half-warp
 // of an odd count at every step. Q^T B, n rows cleared and Q B of 1,000,000 x 8 with 9 / 16
 // columns 1.35 / 1.78 ms (1.99 / 2.02 on the tensor cores, 2 x 1.88 in passes of 8 columns),
 // x 12 with 16 2.52 (2.79), x 16 with 9 2.41 (2.75).
-constexpr int kTileThreads = 256, kTileCols = 16;
+constexpr int kTileThreads = 256, kTileCols = 32;
 
 template <int RM, int MINB>
 __global__ void __launch_bounds__(kTileThreads, MINB) k_apply_tile(const ApplyParamsT<double> p) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int n = p.n, ldt = p.ldt, kc = p.k;
-  double *Bt = reinterpret_cast<double *>(smraw);  // kTileCols columns of ldt rows
-  double *PC = Bt + (size_t)kTileCols * ldt;       // dot products, then update coefficients
+  double *Bt = reinterpret_cast<double *>(smraw);  // kc columns of ldt rows
+  double *PC = Bt + (size_t)kc * ldt;              // dot products, then update coefficients
   double *PV = PC + kTileCols;                     // the pivot row (TSQRT / TTQRT)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, hl = tid & 15;
   TSQR_CHECK_OR_SKIP(p.njobs == 0 || p.job0 + (int)blockIdx.x < p.njobs, p.err)
@@ -467,11 +467,11 @@ __global__ void __launch_bounds__(kTileThreads, MINB) k_apply_tile(const ApplyPa
         load(xn, jn);
         if (do_pf) pf = __ldcg(bp(pr + jn, lane));
       }
-      const int rw = (warp + s) & 7;        // this reflector's pair of columns
-      const int c = 2 * rw + ((tid >> 4) & 1);
-      double *b = Bt + (size_t)c * ldt;
+      const int rw = (warp + s) & 7;        // this reflector's pair of columns of every 16
       const int ra = (hi - lo + 15) >> 4;
-      if (2 * rw < kc) {  // warp-uniform
+      for (int g = 2 * rw; g < kc; g += 16) {  // warp-uniform
+        const int c = g + ((tid >> 4) & 1);
+        const double *b = Bt + (size_t)c * ldt;
         double acc = 0.0;
 #define TSQR_TDOT(r)                                                                        \
   {                                                                                         \
@@ -494,7 +494,9 @@ __global__ void __launch_bounds__(kTileThreads, MINB) k_apply_tile(const ApplyPa
         else *bp(pr + j, lane) = np;
       }
       __syncthreads();
-      if (2 * rw < kc) {
+      for (int g = 2 * rw; g < kc; g += 16) {
+        const int c = g + ((tid >> 4) & 1);
+        double *b = Bt + (size_t)c * ldt;
         const double cf = c < kc ? PC[c] : 0.0;
 #define TSQR_TUPD(r)                                                                        \
   {                                                                                         \
@@ -519,7 +521,7 @@ __global__ void __launch_bounds__(kTileThreads, MINB) k_apply_tile(const ApplyPa
 
 template <int RM, int MINB>
 cudaError_t launch_tile_t(const ApplyParamsT<double> &p, int njobs, cudaStream_t s) {
-  const size_t bytes = sizeof(double) * ((size_t)kTileCols * p.ldt + 2 * kTileCols);
+  const size_t bytes = sizeof(double) * ((size_t)p.k * p.ldt + 2 * kTileCols);
   cudaError_t e = cudaFuncSetAttribute(k_apply_tile<RM, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
   k_apply_tile<RM, MINB><<<njobs, kTileThreads, bytes, s>>>(p);

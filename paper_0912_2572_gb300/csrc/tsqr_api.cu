@@ -616,8 +616,10 @@ static tsqr_status apply_launch(const tsqr_factors *F, double *B, int64_t ldb, i
   const bool narrow = li > 0 && (int64_t)ld.job_count * 4 <= (int64_t)sms * 2;
   // the tile kernel's time grows with n k, the tensor-core kernel's with panels of 8
   // reflectors and groups of 8 columns: they cross at n = 12 with 16 columns 0.90 : 1 (24
-  // columns 1.18), n = 16 with 9 0.88 (16: 1.18), n = 24 with 9 0.95 (16: 1.27)
-  if (kg > 8 && kg <= 16 && !formq && pl.n * kg <= 216) {
+  // columns 1.18), n = 16 with 9 0.88 (16: 1.18), n = 24 with 9 0.95 (16: 1.27); above 16
+  // columns (Q^T B and Q B, 40,000 and 1M rows) n = 4 with 24 0.31 : 0.45 and 1.54 : 2.03 ms,
+  // n = 8 with 17 0.47 : 0.53 and 2.39 : 2.2
+  if (kg > 8 && !formq && (kg <= 16 ? pl.n * kg <= 216 : kg <= 32 && pl.n * kg <= 128)) {
     CUDA_TRY(launch_apply_tile(p, ld.job_count, s));
     return TSQR_OK;
   }

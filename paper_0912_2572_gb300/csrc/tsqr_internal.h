@@ -424,7 +424,7 @@ using ApplyParams = ApplyParamsT<double>;
 // half-warps).
 cudaError_t launch_apply(const ApplyParamsT<double> &p, int njobs, cudaStream_t s, bool tile_pairs = false);
 
-// 9 to 16 columns of B (formq = 0) against few reflectors: one CTA per job (apply.cu).
+// 9 to 32 columns of B (formq = 0) against few reflectors: one CTA per job (apply.cu).
 cudaError_t launch_apply_tile(const ApplyParamsT<double> &p, int njobs, cudaStream_t s);
 
 // More than 8 columns of B: on the tensor cores (apply_mma.cu). rows: the tallest tile of the

@@ -97,3 +97,12 @@ def test_non_finite_columns_stay_alone(cuda_lib, bad):
 ])
 def test_few_reflectors(cuda_lib, m, n, k, h, arity, two):
     test_matches_the_warp_kernel(cuda_lib, m, n, k, h, arity, two)
+
+
+# 17 to 32 columns against fewer reflectors (n k <= 128), and the first widths above
+@pytest.mark.parametrize("m,n,k,h,arity,two", [
+    (129, 4, 32, 128, 0, True), (513, 7, 18, 256, 0, True), (2049, 5, 25, 512, 0, True), (1537, 4, 17, 512, 4, False),
+    (700, 3, 31, 100, 16, False), (600, 5, 26, 257, 0, True), (600, 2, 33, 257, 0, True), (600, 1, 97, 64, 0, True),
+])
+def test_few_reflectors_and_more_columns(cuda_lib, m, n, k, h, arity, two):
+    test_matches_the_warp_kernel(cuda_lib, m, n, k, h, arity, two)
