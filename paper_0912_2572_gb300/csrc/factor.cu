@@ -26,10 +26,9 @@ __device__ int32_t g_error_word;
 
 }  // namespace
 
-size_t cluster_smem_bytes(int n, int nc, size_t optin_per_block) {
+bool cluster_takes(int n, int nc, size_t optin_per_block) {
   const size_t ncp = (size_t)((nc + 7) & ~7);
-  const size_t b = sizeof(double) * ((size_t)nc * n + ncp + (size_t)n * ncp);
-  return b <= optin_per_block ? b : 0;
+  return sizeof(double) * ((size_t)nc * n + ncp + (size_t)n * ncp) <= optin_per_block;
 }
 
 cudaError_t device_error_word(int32_t **ptr) {

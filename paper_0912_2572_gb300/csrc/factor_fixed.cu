@@ -47,11 +47,15 @@ __global__ void __launch_bounds__(32 * NW, 16 / NW) k_factor_fx_cluster(const Fa
   }
 }
 
+size_t cluster_bytes(int n, int nc, int lc, int rpl) {
+  const size_t fx = fx_smem_bytes(n, nc, lc, rpl), f64 = factor_smem_bytes(nc, n, sizeof(double));
+  return fx > f64 ? fx : f64;
+}
+
 template <int CPL, int LC, int RPL, int NW = 8>
 cudaError_t launch_fx_cluster(FactorParamsT<double> p, const ClusterSlot *slots, int nclusters, cudaStream_t s) {
   p.ldt = p.n;  // the combines' tiles: what the shared memory below holds for the FP64 job
-  const size_t fx = fx_smem_bytes(p.n, p.nc, LC, RPL), f64 = factor_smem_bytes(p.nc, p.ldt, sizeof(double));
-  const size_t bytes = fx > f64 ? fx : f64;
+  const size_t bytes = cluster_bytes(p.n, p.nc, LC, RPL);
   cudaError_t e = cudaFuncSetAttribute(k_factor_fx_cluster<CPL, LC, RPL, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)bytes);
   if (e != cudaSuccess) return e;
@@ -128,6 +132,12 @@ cudaError_t launch_factor(const FactorParamsT<double> &p, int njobs, int rows, c
     return launch_fx<2, 4, 18>(p, njobs, s);
   }
   return launch_fx<2, 4, 18, 16>(p, njobs, s);
+}
+
+size_t cluster_smem_bytes(int n, int nc) {
+  if (nc <= 16) return cluster_bytes(n, nc, 1, 2);
+  if (nc <= 32) return cluster_bytes(n, nc, 2, 2);
+  return cluster_bytes(n, nc, 4, nc <= 64 ? 8 : 18);
 }
 
 cudaError_t launch_factor_cluster(const FactorParamsT<double> &p, const ClusterSlot *slots, int nclusters,

@@ -383,11 +383,11 @@ static tsqr_status make_plan_on(const DeviceInfo &di, Plan &pl, int64_t m, int n
   const int64_t chains = chains_override > 0 ? chains_override : (int64_t)di.sms * pl.ctas_per_sm * 4;
   try {
     plan_build(pl, chains);
-    const size_t csm = cluster_smem_bytes(n, nc, di.optin);
-    // resident cluster CTAs per SM: the shared-memory limit, and the register limit (288
-    // threads per CTA at 64 registers, 80 beyond 64 columns: three, two)
-    const int64_t cl_cps = std::min<int64_t>(nc > 64 ? 2 : 3, (int64_t)(di.smem_sm / (csm + di.reserved + 1024)));
-    if ((pl.flags & TSQR_CLUSTER) && pl.arity == 2 && !mixed && csm > 0 && cl_cps >= 1)
+    // resident cluster CTAs per SM: the shared-memory limit, and the build's (two CTAs of 256
+    // threads at 128 registers, one of 512 beyond 64 columns)
+    const size_t csm = cluster_smem_bytes(n, nc);
+    const int64_t cl_cps = std::min<int64_t>(nc > 64 ? 1 : 2, (int64_t)(di.smem_sm / (csm + di.reserved + 1024)));
+    if ((pl.flags & TSQR_CLUSTER) && pl.arity == 2 && !mixed && cluster_takes(n, nc, di.optin) && cl_cps >= 1)
       plan_clusters(pl, (int64_t)di.sms * cl_cps);
     if (max_cps == 2) {
       // batched: the tree works on a compact FP64 array, chain c's pivot block at rows

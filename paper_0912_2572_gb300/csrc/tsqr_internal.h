@@ -236,12 +236,15 @@ constexpr int kClusterSize = 8;
 struct ClusterSlot {
   int32_t job;       // combine job of this CTA, or -1 (idle)
   int32_t child[2];  // cluster rank producing the pivot (0) / tile (1) triangle, or -1 when
-                     // that triangle is complete in global memory (an earlier launch's)
+                     // that triangle is complete in global memory (an earlier launch's); the
+                     // schedule's description (tsqr_plan_clusters), not read on the device
   int32_t round;     // the launch's level (0..2) this combine belongs to
 };
-// Shared memory of a cluster-tier combine CTA (the child's triangle, the dot products and
-// the pivot triangle), 0 when it exceeds the per-block maximum.
-size_t cluster_smem_bytes(int n, int nc, size_t optin_per_block);
+// The widths the tier takes: both triangles of a combine, as doubles, within one CTA's shared
+// memory (the job needs less since its tile is in registers; TSQR_CLUSTER stays ignored beyond).
+bool cluster_takes(int n, int nc, size_t optin_per_block);
+// Shared memory of a cluster-tier combine CTA (factor_fixed.cu).
+size_t cluster_smem_bytes(int n, int nc);
 cudaError_t launch_factor_cluster(const FactorParamsT<double> &p, const ClusterSlot *slots, int nclusters,
                                   cudaStream_t s);
 

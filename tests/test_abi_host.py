@@ -436,3 +436,11 @@ def test_batch_job_table_simulated(lib, chain_tiles, arity):
                 jb = parent
         assert ran == [1] * nj
         assert sorted(finished_items) == list(range(len(items)))
+
+
+@pytest.mark.parametrize("n", [16, 64, 65, 112])
+def test_cluster_launches_fit_one_wave(lib, n):
+    """The first cluster launch's CTAs are resident at once: two per SM up to 64 columns (256
+    threads at 128 registers), one above (512 threads)."""
+    launches, _ = clusters(lib, 1 << 20, n, 144, 0)
+    assert launches and 8 * launches[0][1] <= GB300["sms"] * (2 if n <= 64 else 1)

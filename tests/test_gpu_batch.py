@@ -318,3 +318,26 @@ def test_fp64_items_with_entries_that_are_not_finite(cuda_lib):
         assert np.all(np.isnan(Rb[bad]))
         good = up & ~bad & (np.arange(n)[None, :] < c)
         assert np.linalg.norm((Rb - Ro)[good]) <= 1e-12 * np.linalg.norm(Ro)
+
+
+@pytest.mark.parametrize("n,k", [(72, 0), (90, 5), (96, 0), (96, 1), (128, 1), (128, 15), (120, 24)])
+def test_fp64_items_at_the_edges_of_wide_tiles(cuda_lib, n, k):
+    """The builds of three columns a lane: tiles of 96 rows for 65 to 96 columns, 72 up to 128 (the
+    first width above), 56 above, at and beside their edges, of one to five tiles and with tree
+    nodes in pieces."""
+    import paper_0912_2572_gb300 as ts
+    nc = n + k
+    th = 96 if nc <= 96 else 72 if nc <= 128 else 56
+    items, host = [], []
+    for q, m in enumerate(sorted({max(n, t * th + d) for t in (1, 2, 3, 5) for d in (-1, 0, 1)} | {40 * th + 1})):
+        A, B = inputs.gaussian(m, n, 150 + q), inputs.gaussian(m, max(k, 1), 160 + q)
+        host.append((A, B))
+        items.append({"A": to_dev(A), "prec": ts.FP64, **({"B": to_dev(B)} if k else {})})
+    outs, st = ts.batch_solve(items, chain_tiles=4, status=True)
+    assert st == [0] * len(items)
+    for (A, B), (R, X) in zip(host, outs):
+        Ro = oracle.r_factor(A)
+        assert np.linalg.norm(to_host(R) - Ro) <= 1e-12 * np.linalg.norm(Ro), A.shape
+        if k and A.shape[0] >= 2 * n:  # square problems are as ill-conditioned as their A
+            Xo = oracle.lstsq(A, B)
+            assert np.linalg.norm(to_host(X) - Xo) <= 1e-11 * np.linalg.norm(Xo), A.shape

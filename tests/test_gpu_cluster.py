@@ -126,3 +126,17 @@ def test_cluster_apply_top_down_bitwise(cuda_lib, m, n, k):
     F1.free()
     torch.cuda.synchronize()
     assert ts.error_word() == 0
+
+
+@pytest.mark.parametrize("m,n,h", [(40000, 65, 144), (60000, 112, 144), (30000, 64, 64)])
+def test_cluster_tree_at_the_builds_widths(cuda_lib, m, n, h):
+    """The first and the widest column counts of the one-CTA-per-SM combine, and the last of the
+    two-CTA one: bitwise the per-level tree."""
+    import paper_0912_2572_gb300 as ts
+    A = to_dev(inputs.gaussian(m, n, m + n))
+    R = {}
+    for cl in (False, True):
+        F = ts.factor(A, leaf_h=h, two_level=False, cluster=cl)
+        R[cl] = to_host(F.R)
+        F.free()
+    assert np.array_equal(R[True], R[False])
