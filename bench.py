@@ -49,7 +49,9 @@ FP64_SM_FLOPS_PER_CLK = 4.0   # 2 DFMA per clock per SM on GB300 (measured: 1.20
 # chain: 89.6 with two, because concurrent steps finish together and their copies then
 # queue while the GPU idles; 101.8 with one stream)
 E2E_SLOTS = 4
-CHAIN_DRAM_BYTES_PER_ROW_N64 = (547.427328e6 + 502.893824e6) / 1048576  # ncu, chain launch at m = 1M, n = 64
+# The chain kernel's column steps run on the integer pipe: a 64-bit fixed-point product is three
+# 32 x 32 + 64 bit multiply-adds, one per 2.1 cycles and SM sub-partition (measured, 32 lanes).
+INT_MADS_PER_FMA, INT_MAD_CYCLES = 3, 2.1
 
 
 def flops_step(m, n, k=1):
@@ -1073,6 +1075,7 @@ def bench_ours(args):
     served = None if args.no_serve or rank != 0 else bench_served(ts)
 
     if rank == 0:
+        peak_int = sms * 4 * 32 / (INT_MADS_PER_FMA * INT_MAD_CYCLES) * 2 * 2.07e9 / 1e12
         line = {
             "metric": METRIC, "value": value, "unit": "Gflop/s", "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": t_max / args.steps, "higher_is_better": True,
@@ -1092,16 +1095,19 @@ def bench_ours(args):
                        "apply_qt_ms_beside_form_q": phase_ms.get("apply_qt", 0) / args.steps,
                        "small_ms": phase_ms.get("small", 0) / args.steps},
             "roofline": {"kernel": "k_factor_fx (leaf/flat-chain launch, 64-bit fixed point)", "bound": "alu", "achieved": achieved,
-                         "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                         "traffic": (CHAIN_DRAM_BYTES_PER_ROW_N64 * m if n == 64 else None),
-                         "hbm_gbs": (CHAIN_DRAM_BYTES_PER_ROW_N64 * m / (chain_ms * 1e-3) / 1e9 if n == 64 else None),
+                         "peak": peak_int, "unit": "TFLOP/s", "frac": achieved / peak_int,
+                         "traffic": None, "hbm_gbs": None,
                          "hbm_peak_gbs": measured_hbm_gbs(),
-                         "peak_source": "measured" if peak_measured > 0 else "derived",
-                         "peak_note": f"FP64 DFMA measured live by tsqr_probe_fp64_peak (independent DFMA chains "
+                         "peak_source": "derived",
+                         "peak_note": f"flops of the factorization against the integer multiply-adds it issues: "
+                                      f"{INT_MADS_PER_FMA} per multiply-add, one per {INT_MAD_CYCLES} cycles and SM "
+                                      f"sub-partition (measured), {sms} SMs at 2.07 GHz",
+                         "fp64_pipe_peak": peak, "frac_of_fp64_pipe": achieved / peak,
+                         "fp64_pipe_note": f"FP64 DFMA measured live by tsqr_probe_fp64_peak (independent DFMA chains "
                                       f"on every SM): {peak_measured:.3f} TFLOP/s at {probe_mhz:.0f} MHz; derived {sms} SMs x "
                                       f"{FP64_SM_FLOPS_PER_CLK} flop/clk x 2.07 GHz = {peak_derived:.3f}; the "
                                       "measured-peaks file has no FP64 entry",
-                         "frac_of_derived": achieved / peak_derived,
+                         "frac_of_fp64_pipe_derived": achieved / peak_derived,
                          "fp64_tensor_tflops_measured": dmma_tflops,
                          "fp64_tensor_note": f"DMMA (mma.sync m8n8k4 FP64, tsqr_probe_dmma_peak): {dmma_tflops:.3f} "
                                              f"TFLOP/s at {dmma_mhz:.0f} MHz against the FMA pipe's "

@@ -22,9 +22,19 @@
  *     detected on the host and returned before anything is enqueued.
  *   - The caller owns A, B, R, Q, X. The library owns a tsqr_factors object until
  *     tsqr_free(). A factor set must only be used on the device it was created on.
- *   - Numerical range: entries are squared without rescaling, so matrices with
- *     entries of magnitude above about 1e150 or columns whose squared norms
- *     underflow (below about 1e-300) are outside the supported range.
+ *   - Numerical range: matrices with entries of magnitude above about 1e150, or columns
+ *     whose squared norms underflow (below about 1e-300), are outside the supported range
+ *     (the FP64 jobs square entries without rescaling).
+ *   - Arithmetic of TSQR_FP64: column steps run in FP64 or in 64-bit fixed point, a column
+ *     held as integers at a scale of its own (2^-60 of its norm is one unit), by width and
+ *     height. Fixed point is used where it is no less accurate than FP64: a tile whose
+ *     entries are small beside their column (root mean square below 2^-12 of it, or many
+ *     entries below 2^-16), that is not finite or that has entries outside 2^+-900 goes
+ *     through FP64 with the rest of its chain or node. So rows that differ in scale keep
+ *     their digits where Householder QR in FP64 keeps them (heavy rows first). Q^T B, Q B
+ *     and the thin Q follow the same rule; which arithmetic a call takes depends on n and
+ *     on the number of columns of B, and results of different numbers of columns differ in
+ *     rounding.
  */
 #ifndef TSQR_H
 #define TSQR_H
@@ -46,7 +56,7 @@ typedef enum {
 } tsqr_status;
 
 typedef enum {
-  TSQR_FP64 = 0,  /* every operation in FP64 */
+  TSQR_FP64 = 0,  /* FP64 accuracy throughout (see the arithmetic above) */
   TSQR_MIXED = 1, /* leaf factorizations in FP32 (A rounded on load), tree and
                      refinement in FP64 */
   TSQR_AUTO = 2   /* batch items only: FP64 or MIXED by a cost model (R-only items: FP64) */
@@ -59,13 +69,11 @@ enum {
                          CTA, then the arity-k tree across CTAs (the GPU form of the
                          paper's topology-aware tree, §2.3 and §3) */
   TSQR_CLUSTER = 4    /* with arity 2: the binary tree's levels run three at a time in
-                         thread-block clusters of 8 CTAs, whose combines exchange their
-                         triangles row by row through distributed shared memory and run
-                         as a pipeline (the cluster tier of a hierarchical tree, §2.3 and
-                         §3: CTA -> cluster -> grid). Ignored for other arities or when a
-                         combine's triangles do not fit one CTA's shared memory
-                         (n + extra columns beyond about 80). Same R and reflectors as
-                         the plain binary tree. */
+                         thread-block clusters of 8 CTAs, one launch for three levels with
+                         a cluster barrier between them (the cluster tier of a hierarchical
+                         tree, §2.3 and §3: CTA -> cluster -> grid). Ignored for other
+                         arities and for n + extra columns beyond about 120. Same R and
+                         reflectors as the plain binary tree. */
 };
 
 typedef struct tsqr_factors tsqr_factors; /* opaque factor set */

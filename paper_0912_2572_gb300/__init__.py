@@ -135,8 +135,8 @@ def factor(A, leaf_h: int = 256, arity: int = 2, two_level: bool = True, inplace
     whose ``R`` (n-by-n, diag >= 0) is valid once the stream reaches this point. With
     ``qt`` (an m-by-k column-major tensor), also qt <- Q^T qt, overlapped with the
     factorization's tree (tsqr_factor_qt; not with ``inplace``). ``cluster`` (binary
-    trees) runs the tree's levels three at a time in thread-block clusters, pipelined
-    through distributed shared memory (TSQR_CLUSTER).
+    trees) runs the tree's levels three at a time in thread-block clusters
+    (TSQR_CLUSTER).
     """
     import torch
     lib = _lib.load()

@@ -10,8 +10,12 @@
 // FP32 accumulator holds the sum of digit products of equal weight exactly (4 pairs x 256
 // rows x 2^14 = 2^24), so the 43 digit pairs of weight 256^6 and up take 43 MMA-shares, 5.4
 // cycles per entry and product against 64 (the exact splitting of Ozaki, Ogita, Oishi and
-// Rump, 2012). The 21 pairs left out are below 21 x 2^-21 units of 2^-60 of ||v|| ||c|| a row
-// (24 units in the worst case of 512 rows, signs alike); T is made in FP64.
+// Rump, 2012). The 21 pairs left out are below 0.05 units of 2^-60 of ||v|| ||c|| a row (24
+// units in the worst case of 512 rows, signs alike); T is made in FP64.
+//
+// A tile whose entries are small beside their column, or a reflector with many entries small
+// beside 1, would lose digits at a fixed unit of the column: from there on the job goes through
+// FP64 (apply_rest_fp64). Forward, a column that becomes short is shifted up.
 //
 // A warp holds 8 columns x up to 144 rows of C in registers: lane 4g + t holds column g,
 // rows 8 b + 2t and 8 b + 2t + 1. That is at once the B fragment of V^T C (its digits are cut
@@ -25,10 +29,13 @@
 // Measured on GB300 against the FP64 tile kernel it replaced: thin Q of 4,194,304 x 64
 // 36.3 -> 12.0 ms (chains), Q^T B with 64 columns 16.1 ms, thin Q of 8M x 32 20.7 -> 9.4, of
 // 16M x 16 9.7 -> 7.2 (8 columns 5.2 -> 7.1: those keep the warp kernel); a tree level of one
-// 64-column node 82 -> 50 us. A panel step of a 144 x 64 tile takes 17,600 cycles: V^T C
+// 64-column node 82 -> 50 us. A panel step of a 144 x 64 tile took 17,600 cycles: V^T C
 // 5,000 and the update 7,000 (MMA floor 3,300 and 4,000 for the two warps of a sub-partition),
 // Y 2,000, conversions of the tile 2,800 (an eighth of them each step). Cutting V and making T
-// on the eight main warps and one helper took 24,000.
+// on the eight main warps and one helper took 24,000. The loop is bound by its code, which does
+// not fit the instruction caches (stalls on instruction fetch lead): the checks for small rows
+// and short columns cost Q^T B of 1M x 64 with 32 columns 5.6 -> 7.1 ms, and 29 KB less of it in
+// cut_v gave 6.3 back (thin Q of 1M x 64 5.6, 6.3, 5.7).
 #include <cuda_fp16.h>
 
 #include <algorithm>
